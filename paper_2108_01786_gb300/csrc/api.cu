@@ -236,17 +236,18 @@ __global__ void k_spectral_tables(Blocks B, double2* __restrict__ tw, float2* __
 __global__ void k_rhs(Blocks B, FlowParams F, const double2* __restrict__ z,
                       const double* __restrict__ phit, double* __restrict__ b,
                       long long pstride = 0, long long bstride = 0) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= B.N) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int l = t / OBS_SPLIT, sub = t % OBS_SPLIT;
+  if (l >= B.N) return;           // whole groups leave together
   phit += blockIdx.y * pstride;   // right-hand side blockIdx.y of a batch
   b += blockIdx.y * bstride;
   if (l < B.M[0]) {
-    b[l] = phit[l];
+    if (sub == 0) b[l] = phit[l];
     return;
   }
   const double2 zl = z[l];
-  double v = -F.V1 * zl.y;
-  for (int j = 2; j < F.nb; ++j) {
+  double v = 0.0;
+  for (int j = 2 + sub; j < F.nb; j += OBS_SPLIT) {
     const double ux = zl.x - F.zc[j - 2].x, uy = zl.y - F.zc[j - 2].y;
     double s, c;
     sincos(ux, &s, &c);
@@ -254,7 +255,8 @@ __global__ void k_rhs(Blocks B, FlowParams F, const double2* __restrict__ z,
     const double re = 1.0 - e * c, im = -e * s;
     v += F.a[j - 2] * 0.5 * log(re * re + im * im);   // = -a_j psi_cyl
   }
-  b[l] = v;
+  v = obs_group_sum(v);
+  if (sub == 0) b[l] = v - F.V1 * zl.y;
 }
 
 // App. B right-hand side: b_0 = phi - V1 xi (given), b_k = psi - V1 eta_k on solid nodes
@@ -273,7 +275,7 @@ bie_status rhs_run_many(bie_ctx* c, int nrhs, const double* phit, long long pstr
   const FlowParams F = make_flow(c);
   const double2* z;
   BIE_GET(c, double2, "zeta", c->N, z);
-  k_rhs<<<dim3((c->N + 255) / 256, nrhs), 256, 0, c->stream>>>(B, F, z, phit, b, pstride, bstride);
+  k_rhs<<<dim3(obs_grid(c->N), nrhs), NODE_THREADS, 0, c->stream>>>(B, F, z, phit, b, pstride, bstride);
   BIE_LAUNCH_CHECK(c, "k_rhs");
   return BIE_OK;
 }
@@ -283,7 +285,7 @@ bie_status rhs_run(bie_ctx* c, const double* phit, double* b) {
   const FlowParams F = make_flow(c);
   const double2* z;
   BIE_GET(c, double2, "zeta", c->N, z);
-  k_rhs<<<(c->N + 255) / 256, 256, 0, c->stream>>>(B, F, z, phit, b);
+  k_rhs<<<obs_grid(c->N), NODE_THREADS, 0, c->stream>>>(B, F, z, phit, b);
   BIE_LAUNCH_CHECK(c, "k_rhs");
   return BIE_OK;
 }
@@ -470,7 +472,7 @@ bie_status geometry_prep(bie_ctx* c) {
   BIE_GET(c, double, "T64", c->M[0], T64);
   float2* Tall;
   BIE_GET(c, float2, "Tall", c->N, Tall);
-  const int nthr = 256;
+  const int nthr = NODE_THREADS;
   k_node_prep<<<(unsigned)((ld + nthr - 1) / nthr), nthr, 0, c->stream>>>(
       B, z, dz, d2z, blk, wgt, wgt64, sgn, nP, nQ, nPQc, nZp, nDiag, P64, Q64, diag64, gdiag64, ld);
   BIE_LAUNCH_CHECK(c, "k_node_prep");

@@ -368,6 +368,44 @@ struct FlowParams {
   double2 zc[BIE_MAXB];
 };
 
+// Per-node FP64 kernels (node tables, right-hand side, the multi-valued parts).
+// Bound by FP64 issue: an SM retires two FP64 lanes a cycle, so a warp spends
+// 16 cycles per instruction and a 256-thread CTA of sincos / exp / log chains
+// holds its SM for 10-25 us while most SMs have nothing.  Small CTAs spread the
+// nodes over the whole chip, and OBS_SPLIT lanes share a node's obstacles
+// (at 2944 unknowns and three obstacles k_rhs 19.4 -> 5.7 us, k_velocity_finish_v 19.8 ->
+// 6.9, k_graph_rhs 21.8 -> 8.4, k_node_prep 11.8 -> 7.3 with small CTAs alone).
+#define NODE_THREADS 64
+#define OBS_SPLIT 4
+inline unsigned node_grid(long long n) { return (unsigned)((n + NODE_THREADS - 1) / NODE_THREADS); }
+inline unsigned obs_grid(long long n) { return node_grid(n * OBS_SPLIT); }
+
+// sum over the OBS_SPLIT lanes of a node (a fixed tree; every lane gets it)
+__device__ __forceinline__ double obs_group_sum(double v) {
+  const unsigned lane = threadIdx.x & 31;
+  const unsigned mask = ((1u << OBS_SPLIT) - 1u) << (lane & ~(unsigned)(OBS_SPLIT - 1));
+#pragma unroll
+  for (int o = OBS_SPLIT / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
+}
+
+// sum_j a_j 1/2 cot((z - z_j)/2) over the obstacles, shared by a node's lanes:
+// 1/2 cot(u/2) = i/2 + i/(e^{iu} - 1)
+__device__ __forceinline__ double2 obs_cot_sum(const FlowParams& F, double2 z, int sub) {
+  double re = 0.0, im = 0.0;
+  for (int j = 2 + sub; j < F.nb; j += OBS_SPLIT) {
+    const double ux = z.x - F.zc[j - 2].x, uy = z.y - F.zc[j - 2].y;
+    double s, c;
+    sincos(ux, &s, &c);
+    const double e = exp(-uy);
+    const double qr = e * c - 1.0, qi = e * s;      // e^{iu} - 1
+    const double w = F.a[j - 2] / (qr * qr + qi * qi);
+    re = fma(w, qi, re);
+    im += 0.5 * F.a[j - 2] + w * qr;
+  }
+  return make_double2(obs_group_sum(re), obs_group_sum(im));
+}
+
 inline FlowParams make_flow(const bie_ctx* c) {
   FlowParams f;
   f.nb = c->nb;

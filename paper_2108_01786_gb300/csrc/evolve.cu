@@ -108,19 +108,29 @@ __device__ __forceinline__ double2 dphi_mv(const FlowParams& F, double2 z) {
   return make_double2(re, im);
 }
 
+// the same by the OBS_SPLIT lanes of a node (see obs_cot_sum)
+__device__ __forceinline__ double2 dphi_mv_group(const FlowParams& F, double2 z, int sub) {
+  double asum = 0.0;
+  for (int j = 2; j < F.nb; ++j) asum += F.a[j - 2];
+  const double2 hc = obs_cot_sum(F, z, sub);
+  return make_double2(F.V1 + 0.5 * asum + hc.y, -hc.x);
+}
+
 // eta_t = s U; phi~_t = (phi~_a/s) V + (U - dphi_mv/dn) U - |grad phi|^2/2 - g eta + tau theta_a/s
 __global__ void k_graph_rhs(int M0, FlowParams F, const double2* __restrict__ z,
                             const double2* __restrict__ dz, const double2* __restrict__ d2z,
                             const double* __restrict__ U, const double2* __restrict__ X2,
                             const double* __restrict__ y, double tau, double g,
                             double* __restrict__ ydot) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M0) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = t / OBS_SPLIT, sub = t % OBS_SPLIT;
+  if (m >= M0) return;   // whole groups leave together
+  const double2 dP = dphi_mv_group(F, z[m], sub);
+  if (sub != 0) return;
   const double2 zp = dz[m];
   const double ea = zp.y;
   const double s = sqrt(1.0 + ea * ea);
   const double u = U[m];
-  const double2 dP = dphi_mv(F, z[m]);
   const double dphimv_dn = (-dP.x * zp.y - dP.y * zp.x) / s;   // Re{Phi_mv' i zeta'} / s
   const double phit_a = X2[M0 + m].x / (double)M0;
   const double phi_a = phit_a + (dP.x * zp.x - dP.y * zp.y);  // + Re{Phi_mv' zeta'}
@@ -247,32 +257,46 @@ __global__ void __launch_bounds__(PS_THREADS)
   }
 }
 
-// E = mean_m(tau s + g eta^2 xi_a / 2 + psi_0 phi_a / 2) + sum_j a_j psi_j / 2 (rho = 1), one CTA
-__global__ void k_energy(int M0, FlowParams F, const double2* __restrict__ z,
-                         const double2* __restrict__ dz, const double2* __restrict__ Xd,
-                         const double* __restrict__ psi0, const double* __restrict__ psik,
-                         double tau, double g, double* __restrict__ E) {
-  __shared__ double red[32];
+// E = mean_m(tau s + g eta^2 xi_a / 2 + psi_0 phi_a / 2) + sum_j a_j psi_j / 2 (rho = 1):
+// each CTA leaves the sum over its nodes in part[blockIdx.x], added in order by
+// k_energy_sum (one CTA over all nodes took 97 us at 1472 nodes, the two kernels 12: FP64 issue)
+__global__ void __launch_bounds__(NODE_THREADS)
+    k_energy_part(int M0, FlowParams F, const double2* __restrict__ z,
+                  const double2* __restrict__ dz, const double2* __restrict__ Xd,
+                  const double* __restrict__ psi0, double tau, double g, double* __restrict__ part) {
+  __shared__ double red[NODE_THREADS / 32];
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = t / OBS_SPLIT, sub = t % OBS_SPLIT;
   double acc = 0.0;
-  for (int m = threadIdx.x; m < M0; m += blockDim.x) {
-    const double2 zp = dz[m];
-    const double s = sqrt(zp.x * zp.x + zp.y * zp.y);
-    const double2 dP = dphi_mv(F, z[m]);
-    const double phi_a = Xd[m].x / (double)M0 + (dP.x * zp.x - dP.y * zp.y);
-    const double eta = z[m].y;
-    acc += tau * s + 0.5 * g * eta * eta * zp.x + 0.5 * psi0[m] * phi_a;
+  if (m < M0) {
+    const double2 dP = dphi_mv_group(F, z[m], sub);
+    if (sub == 0) {
+      const double2 zp = dz[m];
+      const double s = sqrt(zp.x * zp.x + zp.y * zp.y);
+      const double phi_a = Xd[m].x / (double)M0 + (dP.x * zp.x - dP.y * zp.y);
+      const double eta = z[m].y;
+      acc = tau * s + 0.5 * g * eta * eta * zp.x + 0.5 * psi0[m] * phi_a;
+    }
   }
+  __syncwarp();
   acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    t = warp_sum(t);
-    if (threadIdx.x == 0) {
-      double e = t / (double)M0;
-      for (int j = 2; j < F.nb; ++j) e += 0.5 * F.a[j - 2] * psik[j - 2];
-      *E = e;
-    }
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < NODE_THREADS / 32; ++w) s += red[w];
+    part[blockIdx.x] = s;
+  }
+}
+__global__ void k_energy_sum(int n, int M0, FlowParams F, const double* __restrict__ part,
+                             const double* __restrict__ psik, double* __restrict__ E) {
+  double t = 0.0;   // one warp
+  for (int i = threadIdx.x; i < n; i += 32) t += part[i];
+  t = warp_sum(t);
+  if (threadIdx.x == 0) {
+    double e = t / (double)M0;
+    for (int j = 2; j < F.nb; ++j) e += 0.5 * F.a[j - 2] * psik[j - 2];
+    *E = e;
   }
 }
 
@@ -346,8 +370,13 @@ bie_status energy_run(bie_ctx* c, const double* phit, const double* omega, doubl
     bie_status s = psi_run(c, omega, psik);
     if (s != BIE_OK) return s;
   }
-  k_energy<<<1, 1024, 0, c->stream>>>(M0, F, z, dz, dX2 + M0, psi0, psik, tau, g, E_dev);
-  BIE_LAUNCH_CHECK(c, "k_energy");
+  const unsigned ge = obs_grid(M0);
+  double* epart;
+  BIE_GET(c, double, "en_part", ge, epart);
+  k_energy_part<<<ge, NODE_THREADS, 0, c->stream>>>(M0, F, z, dz, dX2 + M0, psi0, tau, g, epart);
+  BIE_LAUNCH_CHECK(c, "k_energy_part");
+  k_energy_sum<<<1, 32, 0, c->stream>>>((int)ge, M0, F, epart, psik, E_dev);
+  BIE_LAUNCH_CHECK(c, "k_energy_sum");
   return BIE_OK;
 }
 
@@ -589,7 +618,7 @@ bie_status graph_stage(bie_ctx* c, const double* y, double* ydot, int precision,
     info->max_rel_resid = fmax(info->max_rel_resid, si.rel_resid);
   }
   if (s != BIE_OK) return s;
-  k_graph_rhs<<<(M0 + 255) / 256, 256, 0, c->stream>>>(M0, make_flow(c), z, dz, d2z, sb.U, X2, y,
+  k_graph_rhs<<<obs_grid(M0), NODE_THREADS, 0, c->stream>>>(M0, make_flow(c), z, dz, d2z, sb.U, X2, y,
                                                        tau, g, ydot);
   BIE_LAUNCH_CHECK(c, "k_graph_rhs");
   return BIE_OK;

@@ -123,24 +123,32 @@ __global__ void k_bnd_finish(Blocks B, FlowParams F, int nchunk, const float2* _
                              const double2* __restrict__ d2z64, const int* __restrict__ blk,
                              const float2* __restrict__ gc, const float2* __restrict__ hg,
                              double2* __restrict__ f64, float4* __restrict__ fdf) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= B.N) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = t / OBS_SPLIT, sub = t % OBS_SPLIT;
+  if (m >= B.N) return;   // whole groups leave together
   const int N = B.N;
-  dfl acc[BND_FIELDS];
-  for (int f = 0; f < BND_FIELDS; ++f) acc[f] = {0.f, 0.f};
-  for (int ch = 0; ch < nchunk; ++ch) {
+  // the chunks' partial sums: lane sub takes chunks sub, sub + OBS_SPLIT, ..., added in FP64
+  double acc[BND_FIELDS];
+#pragma unroll
+  for (int f = 0; f < BND_FIELDS; ++f) acc[f] = 0.0;
+  for (int ch = sub; ch < nchunk; ch += OBS_SPLIT) {
     const float2* p = part + (size_t)ch * BND_FIELDS * N;
+#pragma unroll
     for (int f = 0; f < BND_FIELDS; ++f) {
       const float2 v = p[(size_t)f * N + m];
-      acc[f] = acc[f] + dfl{v.x, v.y};
+      acc[f] += (double)v.x + (double)v.y;
     }
   }
-  const double Z0r = df_to_double(acc[0]), Z0i = df_to_double(acc[1]);
-  const double Z1r = df_to_double(acc[2]), Z1i = df_to_double(acc[3]);
-  const double ts = df_to_double(acc[4]);
+#pragma unroll
+  for (int f = 0; f < BND_FIELDS; ++f) acc[f] = obs_group_sum(acc[f]);
+  double asum = 0.0;
+  for (int j = 2; j < F.nb; ++j) asum += F.a[j - 2];
+  const double2 hc = obs_cot_sum(F, z64[m], sub);
+  if (sub != 0) return;
+  const double Z0r = acc[0], Z0i = acc[1], Z1r = acc[2], Z1i = acc[3], ts = acc[4];
   const int k = blk[m];
   const double Mk = (double)B.M[k];
-  const double2 zp = dz64[m], zpp = d2z64[m], zm = z64[m];
+  const double2 zp = dz64[m], zpp = d2z64[m];
   const double cm = df_to_double(dfl{gc[m].x, gc[m].y});
   const double gam = cm * Mk;
   const double hgam = df_to_double(dfl{hg[m].x, hg[m].y});
@@ -158,18 +166,7 @@ __global__ void k_bnd_finish(Blocks B, FlowParams F, int nchunk, const float2* _
     A1i += dim * cm;
   }
   // Phi_mv'(zeta) = V1 + sum_j a_j (1/2 - i 1/2 cot((zeta - z_j)/2))
-  double pr = F.V1, pi = 0.0;
-  for (int j = 2; j < F.nb; ++j) {
-    const double ux = zm.x - F.zc[j - 2].x, uy = zm.y - F.zc[j - 2].y;
-    double s, c;
-    sincos(ux, &s, &c);
-    const double e = exp(-uy);
-    const double qr = e * c - 1.0, qi = e * s;      // e^{iu} - 1
-    const double n2 = qr * qr + qi * qi;
-    const double hr = qi / n2, hi = 0.5 + qr / n2;  // 1/2 cot(u/2) = i/2 + i/q
-    pr += F.a[j - 2] * (0.5 + hi);                  // 1/2 - i (hr + i hi)
-    pi += F.a[j - 2] * (-hr);
-  }
+  const double pr = F.V1 + 0.5 * asum + hc.y, pi = -hc.x;
   const double mvn = -(pr * zp.y + pi * zp.x);      // Re{Phi_mv' i zeta'}
   const double mvs = pr * zp.x - pi * zp.y;         // Re{Phi_mv' zeta'}
   double sn = mvn + A0r + A1i, ss = mvs + A0i - A1r;
@@ -490,7 +487,7 @@ static bie_status boundary_values(bie_ctx* c, const double* omega, double2** f64
   k_bnd_partial<<<dim3((N + 255) / 256, nchunk), 256, 0, c->stream>>>(B, nP, nQ, nPQc, z64, blk, gc,
                                                                      Tall, 0.01f, part);
   BIE_LAUNCH_CHECK(c, "k_bnd_partial");
-  k_bnd_finish<<<(N + 255) / 256, 256, 0, c->stream>>>(B, F, nchunk, part, z64, dz64, d2z64, blk, gc,
+  k_bnd_finish<<<obs_grid(N), NODE_THREADS, 0, c->stream>>>(B, F, nchunk, part, z64, dz64, d2z64, blk, gc,
                                                        hg, f64, fdf);
   BIE_LAUNCH_CHECK(c, "k_bnd_finish");
   *f64_out = f64;
@@ -557,7 +554,7 @@ extern "C" bie_status bie_eval_potential(bie_ctx* c, const double* omega_dev, lo
   if (s != BIE_OK) return s;
   k_c_to_df<<<(N + 255) / 256, 256, 0, c->stream>>>(N, bnd, fdf);
   BIE_LAUNCH_CHECK(c, "k_c_to_df");
-  k_node_weights<<<(N + 255) / 256, 256, 0, c->stream>>>(B, dz64, nEw, hinv2);
+  k_node_weights<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, dz64, nEw, hinv2);
   BIE_LAUNCH_CHECK(c, "k_node_weights");
   k_targets_helsing<<<(unsigned)((n + HEL_TPB - 1) / HEL_TPB), 256, 0, c->stream>>>(
       (int)n, nullptr, nullptr, (const double2*)z_dev, N, nP, nEw, fdf, (double2*)phi_dev);
@@ -597,7 +594,7 @@ extern "C" bie_status bie_eval_velocity(bie_ctx* c, const double* omega_dev, lon
   const float4* nP = (const float4*)ctx_buf(c, "nP", sizeof(float4) * N, &oom);
   const double2* dz64 = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "targets: buffers");
-  k_node_weights<<<(N + 255) / 256, 256, 0, c->stream>>>(B, dz64, nEw, hinv2);
+  k_node_weights<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, dz64, nEw, hinv2);
   BIE_LAUNCH_CHECK(c, "k_node_weights");
   const double2* z = (const double2*)z_dev;
   double2* uv = (double2*)uv_dev;

@@ -351,26 +351,18 @@ __global__ void k_velocity_finish_v(int m0, int m1, long long ld, int npanel, Fl
                                     const double2* __restrict__ z64,
                                     const double2* __restrict__ dz64,
                                     const float2* __restrict__ hw0, double* __restrict__ U) {
-  const int m = m0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= m1) return;
-  double y = 0.0;
-  for (int p = 0; p < npanel; ++p) y += ypart[(size_t)p * ld + m];
-  const double h = df_to_double(dfl{hw0[m].x, hw0[m].y});
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = m0 + t / OBS_SPLIT, sub = t % OBS_SPLIT;
+  if (m >= m1) return;   // whole groups leave together
   const double2 zp = dz64[m];
   double asum = 0.0;
   for (int j = 2; j < F.nb; ++j) asum += F.a[j - 2];
-  double mv = -(F.V1 + 0.5 * asum) * zp.y;
-  const double2 zm = z64[m];
-  for (int j = 2; j < F.nb; ++j) {
-    const double ux = zm.x - F.zc[j - 2].x, uy = zm.y - F.zc[j - 2].y;
-    double s, c;
-    sincos(ux, &s, &c);
-    const double e = exp(-uy);
-    const double qr = e * c - 1.0, qi = e * s;      // e^{iu} - 1
-    const double n2 = qr * qr + qi * qi;
-    const double hr = qi / n2, hi = 0.5 + qr / n2;  // 1/2 cot(u/2) = i/2 + i/q
-    mv += F.a[j - 2] * (hr * zp.x - hi * zp.y);
-  }
+  const double2 hc = obs_cot_sum(F, z64[m], sub);
+  if (sub != 0) return;
+  const double mv = -(F.V1 + 0.5 * asum) * zp.y + (hc.x * zp.x - hc.y * zp.y);
+  double y = 0.0;
+  for (int p = 0; p < npanel; ++p) y += ypart[(size_t)p * ld + m];
+  const double h = df_to_double(dfl{hw0[m].x, hw0[m].y});
   U[m] = (mv + y - 0.5 * h) / hypot(zp.x, zp.y);
 }
 
@@ -460,7 +452,7 @@ bie_status velocity_from_weights(bie_ctx* c, const float2* cw, const float2* hw0
   k_velocity_partial<<<dim3((M0 + 255) / 256, nchunk), 256, 0, c->stream>>>(
       N, M0, nP, nQ, nPQc, z64, blk, cw, Ttab, 0.01f, part);
   BIE_LAUNCH_CHECK(c, "k_velocity_partial");
-  k_velocity_finish<<<(M0 + 255) / 256, 256, 0, c->stream>>>(M0, nchunk, F, part, z64, dz64, gdiag64,
+  k_velocity_finish<<<node_grid(M0), NODE_THREADS, 0, c->stream>>>(M0, nchunk, F, part, z64, dz64, gdiag64,
                                                              cw, hw0, U);
   BIE_LAUNCH_CHECK(c, "k_velocity_finish");
   return BIE_OK;
@@ -539,7 +531,7 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi)
     if (s != BIE_OK) return s;
     const int nv = local_vrows(c);
     if (nv > 0) {
-      k_velocity_finish_v<<<(nv + 255) / 256, 256, 0, c->stream>>>(c->row0, c->row0 + nv, c->ld, npanel,
+      k_velocity_finish_v<<<obs_grid(nv), NODE_THREADS, 0, c->stream>>>(c->row0, c->row0 + nv, c->ld, npanel,
                                                                  F, ypart, z64, dz64, hw0, U);
       BIE_LAUNCH_CHECK(c, "k_velocity_finish_v");
     }
@@ -555,7 +547,7 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi)
   k_velocity_partial<<<dim3((M0 + 255) / 256, nchunk), 256, 0, c->stream>>>(
       N, M0, nP, nQ, nPQc, z64, blk, cw, Ttab, 0.01f, part);
   BIE_LAUNCH_CHECK(c, "k_velocity_partial");
-  k_velocity_finish<<<(M0 + 255) / 256, 256, 0, c->stream>>>(M0, nchunk, F, part, z64, dz64, gdiag64,
+  k_velocity_finish<<<node_grid(M0), NODE_THREADS, 0, c->stream>>>(M0, nchunk, F, part, z64, dz64, gdiag64,
                                                              cw, hw0, U);
   prof_end(c, pr);
   BIE_LAUNCH_CHECK(c, "k_velocity_finish");
@@ -740,7 +732,7 @@ extern "C" bie_status bie_normal_velocity_static(int nb, const int* M_host, cons
   float2* cw = (float2*)(base + L.cw);
   float2* hw0 = (float2*)(base + L.hw0);
   float2* part = (float2*)(base + L.part);
-  k_node_prep<<<(unsigned)((ld + 255) / 256), 256, 0, st>>>(
+  k_node_prep<<<node_grid(ld), NODE_THREADS, 0, st>>>(
       B, z, dz, (const double2*)d2zeta_dev, blk, (float*)(base + L.wgt), (double*)(base + L.wgt64),
       (float*)(base + L.sgn), nP, nQ, nPQc, (float4*)(base + L.nZp), (float2*)(base + L.nDiag),
       (double2*)(base + L.P64), (double2*)(base + L.Q64), (double*)(base + L.diag64), gdiag64, ld);
@@ -776,7 +768,7 @@ extern "C" bie_status bie_normal_velocity_static(int nb, const int* M_host, cons
   const int nchunk = (int)((N + VEL_CH - 1) / VEL_CH);
   k_velocity_partial<<<dim3((M0 + 255) / 256, nchunk), 256, 0, st>>>(
       (int)N, M0, nP, nQ, nPQc, z, blk, cw, Ttab, 0.01f, part);
-  k_velocity_finish<<<(M0 + 255) / 256, 256, 0, st>>>(M0, nchunk, F, part, z, dz, gdiag64, cw, hw0,
+  k_velocity_finish<<<node_grid(M0), NODE_THREADS, 0, st>>>(M0, nchunk, F, part, z, dz, gdiag64, cw, hw0,
                                                       U_dev);
   if (psi_dev && nb > 2) k_psi<<<nb - 2, 256, 0, st>>>(B, omega_dev, psi_dev);
   if (cudaGetLastError() != cudaSuccess) return BIE_ERR_CUDA;
@@ -793,26 +785,19 @@ __global__ void k_pressure_rhs(int N, int M0, FlowParams F, const double2* __res
                                const double2* __restrict__ z64, const double2* __restrict__ dz64,
                                const double2* __restrict__ d2z64, const double* __restrict__ U,
                                double tau, double g, double* __restrict__ b) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= N) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = t / OBS_SPLIT, sub = t % OBS_SPLIT;
+  if (m >= N) return;   // whole groups leave together
   if (m >= M0) {
-    b[m] = 0.0;
+    if (sub == 0) b[m] = 0.0;
     return;
   }
   const double2 z = z64[m], zp = dz64[m], zpp = d2z64[m];
-  double re = F.V1;   // Re Phi_mv'
-  double im = 0.0;    // Im Phi_mv'
-  for (int j = 2; j < F.nb; ++j) {
-    const double ux = z.x - F.zc[j - 2].x, uy = z.y - F.zc[j - 2].y;
-    double sn, cs;
-    sincos(ux, &sn, &cs);
-    const double e = exp(-uy);
-    const double qr = e * cs - 1.0, qi = e * sn;      // e^{iu} - 1
-    const double n2 = qr * qr + qi * qi;
-    const double hr = qi / n2, hi = 0.5 + qr / n2;    // 1/2 cot(u/2) = hr + i hi
-    re += F.a[j - 2] * (0.5 + hi);
-    im -= F.a[j - 2] * hr;
-  }
+  double asum = 0.0;
+  for (int j = 2; j < F.nb; ++j) asum += F.a[j - 2];
+  const double2 hc = obs_cot_sum(F, z, sub);
+  if (sub != 0) return;
+  const double re = F.V1 + 0.5 * asum + hc.y, im = -hc.x;   // Phi_mv'
   const double phia = X2[m].x / (double)M0 + (re * zp.x - im * zp.y);
   const double s2 = zp.x * zp.x + zp.y * zp.y;
   const double s = sqrt(s2);
@@ -859,7 +844,7 @@ extern "C" bie_status bie_pressure_rhs(bie_ctx* c, const double* phit, const dou
   BIE_LAUNCH_CHECK(c, "k_dft_a");
   k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J2, dY, tw, dX2);
   BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_pressure_rhs<<<(N + 255) / 256, 256, 0, c->stream>>>(N, M0, make_flow(c), dX2, z64, dz64, d2z64,
+  k_pressure_rhs<<<obs_grid(N), NODE_THREADS, 0, c->stream>>>(N, M0, make_flow(c), dX2, z64, dz64, d2z64,
                                                          U, tau, g, b);
   BIE_LAUNCH_CHECK(c, "k_pressure_rhs");
   return BIE_OK;
