@@ -264,6 +264,12 @@ struct bie_ctx {
   void* exch_buf = nullptr;      // caller's staging buffer
   size_t exch_bytes = 0;
 
+  // exchange buffers of the one-kernel solver (resident.cu) that were last zeroed
+  const void* rs_bar = nullptr;
+  const void* rs_x = nullptr;
+  long long rs_ld = 0;
+  int rs_n = 0;
+
   // named device buffers
   std::vector<std::pair<std::string, DevBuf>> bufs;
 
@@ -421,6 +427,10 @@ inline FlowParams make_flow(const bie_ctx* c) {
 bie_status asm_run(bie_ctx* c, int precision, int transpose);
 bie_status solve_system(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b,
                         bie_solve_info* info);
+// the solve as one cooperative kernel (resident.cu): enqueue it if it qualifies,
+// then wait for its result
+bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b, bool* taken);
+bie_status resident_result(bie_ctx* c, bie_solve_info* info);
 bie_status gemv_apply(bie_ctx* c, int which, const double* x_dev, double* y_dev);
 bie_status sample_run(bie_ctx* c, int which, long n, const long long* rows, const long long* cols,
                       double* out);

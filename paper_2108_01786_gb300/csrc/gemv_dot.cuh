@@ -15,6 +15,17 @@ template <> struct Dot16<float> {
     acc = fmaf(__uint_as_float(q.w), b.w, acc);
     return acc;
   }
+  // four rows against the same four entries of x
+  static __device__ __forceinline__ void run4(float* acc, const uint4* q, const float* xs) {
+    const float4 b = *reinterpret_cast<const float4*>(xs);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc[i] = fmaf(__uint_as_float(q[i].x), b.x, acc[i]);
+      acc[i] = fmaf(__uint_as_float(q[i].y), b.y, acc[i]);
+      acc[i] = fmaf(__uint_as_float(q[i].z), b.z, acc[i]);
+      acc[i] = fmaf(__uint_as_float(q[i].w), b.w, acc[i]);
+    }
+  }
 };
 template <> struct Dot16<__half> {
   static constexpr int E = 8;
@@ -35,6 +46,27 @@ template <> struct Dot16<__half> {
     acc = fmaf(f.x, b1.z, acc);
     acc = fmaf(f.y, b1.w, acc);
     return acc;
+  }
+  // four rows against the same eight entries of x
+  static __device__ __forceinline__ void run4(float* acc, const uint4* q, const float* xs) {
+    const float4 b0 = *reinterpret_cast<const float4*>(xs);
+    const float4 b1 = *reinterpret_cast<const float4*>(xs + 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float2 f;
+      f = __half22float2(*reinterpret_cast<const __half2*>(&q[i].x));
+      acc[i] = fmaf(f.x, b0.x, acc[i]);
+      acc[i] = fmaf(f.y, b0.y, acc[i]);
+      f = __half22float2(*reinterpret_cast<const __half2*>(&q[i].y));
+      acc[i] = fmaf(f.x, b0.z, acc[i]);
+      acc[i] = fmaf(f.y, b0.w, acc[i]);
+      f = __half22float2(*reinterpret_cast<const __half2*>(&q[i].z));
+      acc[i] = fmaf(f.x, b1.x, acc[i]);
+      acc[i] = fmaf(f.y, b1.y, acc[i]);
+      f = __half22float2(*reinterpret_cast<const __half2*>(&q[i].w));
+      acc[i] = fmaf(f.x, b1.z, acc[i]);
+      acc[i] = fmaf(f.y, b1.w, acc[i]);
+    }
   }
 };
 template <> struct Dot16<__nv_bfloat16> {
@@ -57,6 +89,27 @@ template <> struct Dot16<__nv_bfloat16> {
     acc = fmaf(f.y, b1.w, acc);
     return acc;
   }
+  // four rows against the same eight entries of x
+  static __device__ __forceinline__ void run4(float* acc, const uint4* q, const float* xs) {
+    const float4 b0 = *reinterpret_cast<const float4*>(xs);
+    const float4 b1 = *reinterpret_cast<const float4*>(xs + 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float2 f;
+      f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q[i].x));
+      acc[i] = fmaf(f.x, b0.x, acc[i]);
+      acc[i] = fmaf(f.y, b0.y, acc[i]);
+      f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q[i].y));
+      acc[i] = fmaf(f.x, b0.z, acc[i]);
+      acc[i] = fmaf(f.y, b0.w, acc[i]);
+      f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q[i].z));
+      acc[i] = fmaf(f.x, b1.x, acc[i]);
+      acc[i] = fmaf(f.y, b1.y, acc[i]);
+      f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q[i].w));
+      acc[i] = fmaf(f.x, b1.z, acc[i]);
+      acc[i] = fmaf(f.y, b1.w, acc[i]);
+    }
+  }
 };
 
 // s + (ah + al)(xh + xl) in double-float (the al xl term is below the precision)
@@ -69,3 +122,30 @@ __device__ __forceinline__ dfl df_acc_prod(dfl s, float ah, float al, float xh, 
   return df_fast_two_sum(t.hi, lo);
 }
 
+
+// A sum kept as three floats (about 72 bits): the flush target of short
+// double-float runs.  FP64 accumulators cost 4 FP64 instructions per flush, 64
+// cycles of an SM's FP64 pipe per warp, which is what bound the hi + lo products
+// whose matrix sits in L2; these are ~20 FP32 instructions (5 cycles).
+struct tfl {
+  float s, e, f;
+};
+__device__ __forceinline__ void tf_add(tfl& a, float h, float l) {
+  const dfl t = df_two_sum(a.s, h);
+  const dfl u = df_two_sum(a.e, l);
+  const dfl w = df_two_sum(u.hi, t.lo);
+  a.s = t.hi;
+  a.e = w.hi;
+  a.f += u.lo + w.lo;
+}
+__device__ __forceinline__ tfl tf_warp_sum(tfl a) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float s = __shfl_xor_sync(0xffffffffu, a.s, o), e = __shfl_xor_sync(0xffffffffu, a.e, o);
+    const float f = __shfl_xor_sync(0xffffffffu, a.f, o);
+    tf_add(a, s, e);
+    a.f += f;
+  }
+  return a;
+}
+__device__ __forceinline__ double tf_to_double(tfl a) { return (double)a.s + ((double)a.e + (double)a.f); }

@@ -1186,6 +1186,10 @@ static bie_status run_solver(bie_ctx* c, const bie_solve_opts* o, double* x, con
 
 bie_status solve_system(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b,
                         bie_solve_info* info) {
+  bool taken = false;
+  const bie_status s = resident_launch(c, o, x, b, &taken);
+  if (s != BIE_OK) return s;
+  if (taken) return resident_result(c, info);
   return (c->precision == BIE_FP64) ? run_solver<double>(c, o, x, b, info)
                                     : run_solver<float>(c, o, x, b, info);
 }
@@ -1196,6 +1200,14 @@ bie_status solve_run(bie_ctx* c, const double* phit, double* omega, double* U, d
   BIE_GET(c, double, "kr_b", c->ld, b);
   bie_status s = rhs_run(c, phit, b);
   if (s != BIE_OK) return s;
+  bool taken = false;
+  s = resident_launch(c, o, omega, b, &taken);
+  if (s != BIE_OK) return s;
+  if (taken) {   // U goes in behind the solve, one wait for both
+    s = velocity_run(c, omega, U, psi);
+    if (s != BIE_OK) return s;
+    return resident_result(c, info);
+  }
   bie_status ss = (c->precision == BIE_FP64) ? run_solver<double>(c, o, omega, b, info)
                                              : run_solver<float>(c, o, omega, b, info);
   if (ss != BIE_OK && ss != BIE_ERR_NOCONV) return ss;

@@ -1,0 +1,117 @@
+"""The one-kernel solver (csrc/resident.cu) against the kernel-by-kernel one,
+which profiling selects, at the sizes where its row split can go wrong: one CTA,
+one row more or less than the row warps take, row counts per CTA off the quads,
+all SMs; restart lengths from 1, no obstacles and many, both row signs, initial
+guesses, zero and non-finite data.
+
+Both stop at ||r|| <= 1e-14 ||b|| (the caller's rtol where it is larger), so their
+solutions differ by at most 2 rtol ||b|| / sigma_min(A) plus rounding; sigma_min >=
+0.1 ||A|| on these geometries (spectrum clustered at 1/2): 1e-12 of ||omega|| bounds
+it for rtol 1e-14, 100 rtol in general."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_2108_01786_gb300 as P
+    from paper_2108_01786_gb300 import _build
+    _build.build()
+    return P
+
+
+def _geometry(M0, M1, Mo):
+    surf = W.fourier_graph(M0, 0.0, np.array([0.08, 0.02]), np.array([0.03, 0.0]))
+    bot = W.graph_curve(M1, lambda a: -1.0 + 0 * a, lambda a: 0 * a, lambda a: 0 * a)
+    n = max(1, len(Mo))
+    ells = [(6.28 * (j + 0.5) / n, -0.5 - 0.01 * j, 0.12, 0.1, 0.4 * j) for j in range(len(Mo))]
+    g = W.assemble_geometry([surf, bot] + [W.ellipse(m, *e) for m, e in zip(Mo, ells)], ells)
+    a = np.linspace(-0.4, 0.5, len(Mo)) if Mo else np.zeros(0)
+    return g, W.Flow(V1=0.7, a=a), W.filtered_noise(np.random.default_rng(M0), M0, 0.05, min(8, M0 // 4))
+
+
+SIZES = [(16, 12, []),                      # one CTA, fewer rows than a quad round
+         (20, 11, []),                      # 31 rows: one CTA, every row warp
+         (20, 12, []),                      # 32: two CTAs
+         (41, 29, [23, 25]),                # 118 rows on 4 CTAs, the last one short
+         (150, 81, [40] * 6),               # six obstacles
+         (640, 330, [161, 170]),            # 1301 rows
+         (2356, 1178, [589, 589]),          # 31 x 152: one row per row warp on every SM
+         (2357, 1179, [589, 589])]          # and two more rows
+
+
+@pytest.mark.parametrize("M0,M1,Mo", SIZES)
+@pytest.mark.parametrize("prec", ["fp64", "fp32_ir", "fp16_ir", "bf16_ir"])
+def test_one_kernel_solve_equals_the_stepwise_one(P, M0, M1, Mo, prec):
+    import torch
+    g, f, ph = _geometry(M0, M1, Mo)
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        rng = np.random.default_rng(3)
+        b = torch.as_tensor(np.concatenate([W.filtered_noise(rng, m, 0.5, max(1, m // 8)) for m in g.M]), device="cuda")
+        for kw in ({}, {"row_flip": 0}, {"restart": 3, "max_cycles": 60, "rtol": 1e-12}, {"restart": 1, "rtol": 1e-4},
+                   {"restart": 200}, {"rtol": 1e-10, "inner_tol": 1e-2}):
+            o = P.bie_default_opts(**kw)
+            res = []
+            for prof in (0, 1):
+                P.bie_set_profiling(prob.ctx, prof)
+                om = torch.full((g.N,), np.nan, dtype=torch.float64, device="cuda")
+                try:
+                    info, st = P.bie_solve_b(prob.ctx, b, om, o), 0
+                except P.BieError as e:
+                    info, st = None, e.status
+                res.append((st, om.cpu().numpy(), info))
+            (s0, x0, i0), (s1, x1, i1) = res
+            assert s0 == s1, (kw, s0, s1)
+            if s0 == 0:
+                assert i0.converged and i0.rel_resid <= o.rtol
+                bound = max(1e-12, 100.0 * o.rtol)
+                assert np.linalg.norm(x0 - x1) <= bound * np.linalg.norm(x1), kw
+    finally:
+        prob.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_ir", "fp16_ir"])
+def test_one_kernel_solve_guesses_zero_and_nonfinite(P, prec):
+    import torch
+    g, f, ph = _geometry(120, 61, [40, 41])
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        prob.solve()
+        om = prob.omega.clone()
+        # from the solution: nothing to do; from a perturbed one: the same solution
+        assert P.bie_solve(prob.ctx, prob.phit, prob.omega, prob.U, None, P.bie_default_opts(x0=1)).cycles <= 1
+        prob.omega.copy_(om * (1.0 + 1e-3) + 1e-4)
+        info = P.bie_solve(prob.ctx, prob.phit, prob.omega, prob.U, None, P.bie_default_opts(x0=1))
+        assert info.converged
+        assert float((prob.omega - om).norm() / om.norm()) <= 1e-12
+        z = torch.zeros(g.N, dtype=torch.float64, device="cuda")
+        for x0 in (0, 1):
+            x = torch.ones(g.N, dtype=torch.float64, device="cuda")
+            info = P.bie_solve_b(prob.ctx, z, x, P.bie_default_opts(x0=x0))
+            assert info.converged and info.iters == 0 and float(x.abs().max()) == 0.0
+        z[7] = float("nan")
+        with pytest.raises(P.BieError) as e:
+            P.bie_solve_b(prob.ctx, z, x)
+        assert e.value.status == P.BIE_ERR_NAN
+        with pytest.raises(P.BieError) as e:
+            P.bie_solve(prob.ctx, prob.phit, prob.omega, prob.U, None, P.bie_default_opts(max_cycles=1, restart=2))
+        assert e.value.status == P.BIE_ERR_NOCONV
+        assert prob.solve().converged   # the context stays usable
+        # tiny and huge data (the solve is linear)
+        for s in (1e-30, 1e30):
+            info = P.bie_solve(prob.ctx, prob.phit, prob.omega, prob.U, None)
+            b = torch.empty(g.N, dtype=torch.float64, device="cuda")
+            P.bie_rhs(prob.ctx, prob.phit, b)
+            x = torch.empty_like(b)
+            info = P.bie_solve_b(prob.ctx, b * s, x)
+            assert info.converged
+            assert float((x / s - prob.omega).norm() / prob.omega.norm()) <= 1e-12
+    finally:
+        prob.close()
