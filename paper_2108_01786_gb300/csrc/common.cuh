@@ -76,9 +76,11 @@ __device__ __forceinline__ dfl df_addf(dfl a, float b) {
 }
 // Reciprocal by one Newton step (with its second-order term) from the
 // hardware approximation: r0 ~ 1/b, e = 1 - b r0, 1/b = r0 (1 + e + e^2 + ...).
+// (ftz: without it the compiler wraps the instruction in a subnormal test and two
+// scalings; |d|^2 and |Delta E|^2 of distinct nodes are normal numbers)
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 __device__ __forceinline__ dfl df_rcp(dfl b) {

@@ -91,8 +91,8 @@ __device__ __forceinline__ df2 d2_dot2(df2 a, df2 b, df2 c, df2 d, float2 khi, f
 // second-order term, e = 1 - b r, 1/b = r (1 + e + e^2 + ...)
 __device__ __forceinline__ df2 d2_rcp(df2 b) {
   float2 r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r.x) : "f"(b.hi.x));
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r.y) : "f"(b.hi.y));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(b.hi.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(b.hi.y));
   float2 e = p_fma(p_neg(b.hi), r, f2(1.f));
   e = p_fma(p_neg(b.lo), r, e);
   const float2 re = p_mul(r, e);

@@ -15,12 +15,14 @@
 // step of eq. plemelj:ver2), a matrix-free pass over M_0 x N node pairs with
 // the assembly's double-float kernel G = 1/2 cot((zeta_l - zeta_m)/2).
 #include <cmath>
+#include <algorithm>
 #include <cstring>
 #include <vector>
 #include "common.cuh"
 #include "nvtx.cuh"
 #include "dft.cuh"
 #include "pair_kernel.cuh"
+#include "pair_sums.cuh"
 
 namespace {
 
@@ -207,45 +209,110 @@ __device__ __forceinline__ dfl df_cta_sum(dfl v, dfl* sh) {
   return t;
 }
 
-// psi on the surface, one 128-thread CTA per row m: the sums of the file
-// comment with the double-float pair kernel of the assembly (separable far
-// field, FP64 node differences near the diagonal); the diagonal term in FP64.
-// w = omega_l / M_j as double-float.
-__global__ void __launch_bounds__(PS_THREADS)
-    k_psi_surface(Blocks B, PairNodes nd, const double2* __restrict__ dz,
-                  const double2* __restrict__ d2z, const float2* __restrict__ w,
-                  const double* __restrict__ omega, const double2* __restrict__ Hx, FlowParams F,
-                  double* __restrict__ psi0) {
-  __shared__ dfl sh[PS_THREADS / 32];
-  const int M0 = B.M[0], N = B.N;
-  const int m = blockIdx.x;
-  const cx<dfl> Qm = ld_cx(nd.nQ, m);
-  const float4 qc = nd.nPQc[m];
-  const float2 Qcm = make_float2(qc.z, qc.w);
-  const double2 zm = nd.z64[m];
+// The component of Phi~ on the boundaries that is not a row of eq. lin:sys, over
+// a chunk of sources l != m (see pair_sums.cuh), with W_l = zeta_l' omega_l / M_j
+// and G = 1/2 cot((zeta_l - zeta_m)/2):
+//   surface target (psi):      -[Re{W G} - T w] on surface columns, Im{W G} on solid ones
+//   solid target (Re Phi~):     Im{W G} on surface columns, Re{W G} on solid ones,
+//                               less T w on its own boundary
+// (T = 1/2 cot((beta_l - alpha_m)/2)); targets m < m_hi (the surface or every
+// node), the sum over split c of the sources at part[c m_hi + m].  One CTA per
+// target with the general pair kernel took 318 us for 6001 nodes, this 214 us.
+__global__ void __launch_bounds__(PSUM_THREADS, 3)
+    k_pot_partial(Blocks B, PsumNodes nd, int ntile, const float4* __restrict__ nZp,
+                  const float2* __restrict__ w, int m_hi, float2* __restrict__ part) {
+  __shared__ PsumStage<3> S[PSUM_WARPS];
+  __shared__ PsumClose<3> sc[PSUM_WARPS];
+  __shared__ unsigned mask[PSUM_MAXTILES / 32 + 1];
+  __shared__ dfl red[PSUM_WARPS][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int km, m0, mn;
+  psum_tile(B, blockIdx.x, km, m0, mn);
+  const int m = m0 + min(lane, mn - 1);
+  PsumTarget T;
+  T.load(nd, m);
+  const float4 tbox = psum_box(T.z);
+  const int om = B.off[km], Mk = B.M[km], im = m - om;
+  auto weights = [&](int l, dfl* v) {
+    const cx<dfl> Z = ld_cx(nZp, l);
+    v[2] = {w[l].x, w[l].y};
+    v[0] = Z.re * v[2];
+    v[1] = Z.im * v[2];
+  };
   dfl acc = {0.f, 0.f};
-  for (int l = threadIdx.x; l < N; l += PS_THREADS) {
-    if (l == m) continue;   // diagonal added below in FP64
-    const float4 pc = nd.nPQc[l];
-    const cx<dfl> G = half_cot_pair<dfl>(ld_cx(nd.nP, l), Qm, make_float2(pc.x, pc.y), Qcm,
-                                         nd.z64[l], zm, 0.01f);
-    const cx<dfl> Zl = ld_cx(nd.nZp, l);
-    const dfl wl = {w[l].x, w[l].y};
-    if (l < M0) {
-      const float2 t = nd.Ttab[(l - m + M0) % M0];
-      acc = acc - (cre(Zl, G) - dfl{t.x, t.y}) * wl;
-    } else {
-      acc = acc + cim(Zl, G) * wl;
+  auto stage = [&](int sl, int l0, int n, dfl* ws) -> bool {
+    float4 sbox;
+    psum_stage<3>(S[sl], nd, l0, n, weights, ws, sbox);
+    return !psum_apart(tbox, sbox);
+  };
+  auto work = [&](int sl, int kl, int l0, int n, const dfl* ws, int p0, int p1, bool close, bool own) {
+    const bool same = kl == km, re = (kl == 0) == (km == 0);
+    int idx = (l0 - om) - im;               // (i_l - i_m) mod M_k of the tile's first source
+    if (same && idx < 0) idx += Mk;
+    df2 a2 = {f2(0.f), f2(0.f)}, at = a2;
+#pragma unroll 1
+    for (int p = p0; p < p1; ++p) {
+      df2 dr, di, inv;
+      psum_pair(S[sl], p, nd, T, close, l0, n, m, dr, di, inv);
+      const df2 Wr = d2_of(S[sl].W[0][p]), Wi = d2_of(S[sl].W[1][p]);
+      // W i/d = (Wr + i Wi)(di + i dr) inv
+      const df2 v = re ? d2_dot2<false>(Wr, di, d2_neg(Wi), dr, f2(0.f), f2(0.f))
+                       : d2_dot2<false>(Wr, dr, Wi, di, f2(0.f), f2(0.f));
+      a2 = d2_macc(a2, v, inv);
+      if (same) {   // T_0 = 0: the target itself drops out
+        int ia = idx + p;
+        ia -= ia >= Mk ? Mk : 0;
+        int ib = ia + 16;
+        ib -= ib >= Mk ? Mk : 0;
+        const float2 ta = nd.Tall[om + ia], tb = nd.Tall[om + ib];
+        at = d2_macc(at, df2{f2(ta.x, tb.x), f2(ta.y, tb.y)}, d2_of(S[sl].W[2][p]));
+      }
     }
+    dfl v = d2_fold(a2);
+    if (same) v = v - d2_fold(at);
+    if (own) {   // the i/2 of G: Re -W.im/2, Im W.re/2, without the target's own
+      v = v + (re ? -df_half(ws[1]) : df_half(ws[0]));
+      if (same && m >= l0 && m < l0 + n) {
+        dfl self[3];
+        weights(m, self);
+        v = v + df_half(self[1]);
+      }
+    }
+    acc = (re && km == 0) ? acc - v : acc + v;
+  };
+  psum_tiles<3>(B, ntile, sc, mask, stage, work);
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && lane < mn) {
+    dfl v = red[0][lane];
+    for (int k = 1; k < PSUM_WARPS; ++k) v = v + red[k][lane];
+    part[(size_t)blockIdx.y * m_hi + m0 + lane] = make_float2(v.hi, v.lo);
   }
-  acc = df_cta_sum(acc, sh);
-  if (threadIdx.x == 0) {
-    const double2 a = d2z[m], b = dz[m];
-    const double n2 = b.x * b.x + b.y * b.y;
-    double tot = (double)acc.hi + (double)acc.lo -
-                 0.5 * (a.x * b.x + a.y * b.y) / n2 * omega[m] / (double)M0;
-    double pm = F.V1 * zm.y;
-    for (int j = 2; j < F.nb; ++j) {
+}
+
+// The chunks' sums, the diagonal limit zeta''/(2 zeta') and the Hilbert term in
+// FP64: psi0 on the surface targets (psi_mv of F added), the real part of out on the
+// solid ones.  Hx holds M_k H omega_k.
+__global__ void k_pot_finish(Blocks B, int nchunk, int m_hi, FlowParams F,
+                             const float2* __restrict__ part, const double2* __restrict__ z,
+                             const double2* __restrict__ dz, const double2* __restrict__ d2z,
+                             const double* __restrict__ omega, const double2* __restrict__ Hx,
+                             double* __restrict__ psi0, double2* __restrict__ out) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = g / OBS_SPLIT, sub = g % OBS_SPLIT;
+  if (m >= m_hi) return;   // whole groups leave together
+  dfl acc = {0.f, 0.f};
+#pragma unroll 4
+  for (int ch = sub; ch < nchunk; ch += OBS_SPLIT) {
+    const float2 v = part[(size_t)ch * m_hi + m];
+    acc = acc + dfl{v.x, v.y};
+  }
+  const double tot = obs_group_sum(df_to_double(acc));
+  const double2 zm = z[m];
+  const bool surf = m < B.M[0];
+  double pm = 0.0;
+  if (surf)
+    for (int j = 2 + sub; j < F.nb; j += OBS_SPLIT) {
       const double ux = zm.x - F.zc[j - 2].x, uy = zm.y - F.zc[j - 2].y;
       double sn, cs;
       sincos(ux, &sn, &cs);
@@ -253,8 +320,15 @@ __global__ void __launch_bounds__(PS_THREADS)
       const double re = 1.0 - e * cs, im = -e * sn;
       pm -= F.a[j - 2] * 0.5 * log(re * re + im * im);   // a_j psi_cyl, psi_cyl = -ln|1 - e^{iz}|
     }
-    psi0[m] = 0.5 * Hx[m].x / (double)M0 + tot + pm;
-  }
+  pm = obs_group_sum(pm);
+  if (sub != 0) return;
+  const double2 a = d2z[m], b = dz[m];
+  const double diag = 0.5 * (a.x * b.x + a.y * b.y) / (b.x * b.x + b.y * b.y);
+  int k = 0;
+  while (k + 1 < B.nb && m >= B.off[k + 1]) ++k;
+  const double Mk = (double)B.M[k];
+  if (surf) psi0[m] = 0.5 * Hx[m].x / Mk + (tot - diag * omega[m] / Mk) + (pm + F.V1 * zm.y);
+  else out[m].x = tot + diag * omega[m] / Mk - 0.5 * Hx[m].x / Mk;
 }
 
 // E = mean_m(tau s + g eta^2 xi_a / 2 + psi_0 phi_a / 2) + sum_j a_j psi_j / 2 (rho = 1):
@@ -298,6 +372,29 @@ __global__ void k_energy_sum(int n, int M0, FlowParams F, const double* __restri
     for (int j = 2; j < F.nb; ++j) e += 0.5 * F.a[j - 2] * psik[j - 2];
     *E = e;
   }
+}
+
+// k_pot_partial and k_pot_finish for the surface nodes, or for every node
+bie_status pot_run(bie_ctx* c, bool all, const FlowParams& F, const PairNodes& nd, const float2* w,
+                   const double* omega, const double2* Hx, double* psi0, double2* out) {
+  const int N = c->N, m_hi = all ? N : c->M[0];
+  const Blocks B = make_blocks(c);
+  const int ntile = psum_ntile(B), nt = all ? ntile : psum_ntile0(B);
+  const int nch = psum_nsplit(nt, ntile);
+  float2* part;
+  BIE_GET(c, float2, "pot_part", (size_t)nch * m_hi, part);
+  bool oom = false;
+  const double2* dz = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
+  const double2* d2z = (const double2*)ctx_buf(c, "d2zeta", sizeof(double2) * N, &oom);
+  const float2* Tall = (const float2*)ctx_buf(c, "Tall", sizeof(float2) * N, &oom);
+  if (oom) return ctx_fail(c, BIE_ERR_OOM, "boundary sums: buffers");
+  const PsumNodes pn = {nd.nP, nd.nQ, nd.nPQc, nd.z64, Tall};
+  k_pot_partial<<<dim3(nt, nch), PSUM_THREADS, 0, c->stream>>>(B, pn, ntile, nd.nZp, w, m_hi, part);
+  BIE_LAUNCH_CHECK(c, "k_pot_partial");
+  k_pot_finish<<<obs_grid(m_hi), NODE_THREADS, 0, c->stream>>>(B, nch, m_hi, F, part, nd.z64, dz, d2z, omega,
+                                                               Hx, psi0, out);
+  BIE_LAUNCH_CHECK(c, "k_pot_finish");
+  return BIE_OK;
 }
 
 }  // namespace
@@ -359,11 +456,12 @@ bie_status energy_run(bie_ctx* c, const double* phit, const double* omega, doubl
   const Blocks B = make_blocks(c);
   const FlowParams F = make_flow(c);
   float2* wdf;
+  bie_status s_pot;
   BIE_GET(c, float2, "en_wdf", N, wdf);
   k_to_df<<<(N + 255) / 256, 256, 0, c->stream>>>(B, N, omega, 1, wdf);
   BIE_LAUNCH_CHECK(c, "k_to_df");
-  k_psi_surface<<<M0, PS_THREADS, 0, c->stream>>>(B, nd, dz, d2z, wdf, omega, dX2, F, psi0);
-  BIE_LAUNCH_CHECK(c, "k_psi_surface");
+  s_pot = pot_run(c, false, F, nd, wdf, omega, dX2, psi0, nullptr);
+  if (s_pot != BIE_OK) return s_pot;
   // psi_j = <1_j, omega> for obstacles (eq. psi:k)
   BIE_CUDA_TRY(c, cudaMemsetAsync(psik, 0, sizeof(double) * BIE_MAXB, c->stream));
   if (c->nb > 2) {
@@ -1305,58 +1403,6 @@ bie_status step_drive(bie_ctx* c, StageFn stage, StepFn step, const char* who, d
   return BIE_OK;
 }
 
-// Re Phi~ on the solid boundaries from the fluid side: the Plemelj formula
-// applied to eq. w123 (Sec. 4: Phi_t - C on the boundaries).  The jump
-// (i/2) omega_k of the own boundary is imaginary and drops out; one CTA per
-// solid node m (boundary k >= 1), double-float sums over every source l of
-//   Im{zeta_l' G} on surface columns, Re{zeta_l' G} on the other solid
-//   boundaries, Re{zeta_l' G} - 1/2 cot((beta_l - alpha_m)/2) on boundary k,
-// each times omega_l / M_j (G = 1/2 cot((zeta_l - zeta_m)/2)); then the
-// diagonal limit Re{zeta''/(2 zeta')} omega_m / M_k and -(1/2) H omega_k (the
-// principal value of the subtracted cotangent) in FP64.  Hb holds M_k H omega_k.
-__global__ void __launch_bounds__(PS_THREADS)
-    k_phi_solid(Blocks B, PairNodes nd, const float2* __restrict__ Tall,
-                const double2* __restrict__ dz, const double2* __restrict__ d2z,
-                const float2* __restrict__ w, const double* __restrict__ omega,
-                const double2* __restrict__ Hb, double2* __restrict__ out) {
-  __shared__ dfl sh[PS_THREADS / 32];
-  const int M0 = B.M[0], N = B.N;
-  const int m = M0 + (int)blockIdx.x;
-  int k = 1;
-  while (k + 1 < B.nb && m >= B.off[k + 1]) ++k;
-  const int ok = B.off[k], Mk = B.M[k];
-  const cx<dfl> Qm = ld_cx(nd.nQ, m);
-  const float4 qc = nd.nPQc[m];
-  const float2 Qcm = make_float2(qc.z, qc.w);
-  const double2 zm = nd.z64[m];
-  dfl acc = {0.f, 0.f};
-  for (int l = threadIdx.x; l < N; l += PS_THREADS) {
-    if (l == m) continue;   // diagonal added below in FP64
-    const float4 pc = nd.nPQc[l];
-    const cx<dfl> G = half_cot_pair<dfl>(ld_cx(nd.nP, l), Qm, make_float2(pc.x, pc.y), Qcm,
-                                         nd.z64[l], zm, 0.01f);
-    const cx<dfl> Zl = ld_cx(nd.nZp, l);
-    const dfl wl = {w[l].x, w[l].y};
-    if (l < M0) {
-      acc = acc + cim(Zl, G) * wl;
-    } else if (l >= ok && l < ok + Mk) {
-      int d = l - m;
-      if (d < 0) d += Mk;
-      const float2 t = Tall[ok + d];
-      acc = acc + (cre(Zl, G) - dfl{t.x, t.y}) * wl;
-    } else {
-      acc = acc + cre(Zl, G) * wl;
-    }
-  }
-  acc = df_cta_sum(acc, sh);
-  if (threadIdx.x == 0) {
-    const double2 a = d2z[m], b = dz[m];
-    const double diag = 0.5 * (a.x * b.x + a.y * b.y) / (b.x * b.x + b.y * b.y);
-    out[m].x = (double)acc.hi + (double)acc.lo + diag * omega[m] / (double)Mk -
-               0.5 * Hb[m].x / (double)Mk;
-  }
-}
-
 // The parts of Phi~ on the boundaries that the operator of eq. lin:sys and the
 // energy's psi give: Re on Gamma_0 = (A omega)_m, Im on Gamma_0 = psi_0 without
 // psi_mv, Im on Gamma_k = (A omega)_m, plus <1_k, omega> on obstacles (the term
@@ -1412,13 +1458,10 @@ bie_status boundary_potential_run(bie_ctx* c, const double* omega, double2* out)
   BIE_LAUNCH_CHECK(c, "k_to_df");
   FlowParams F0 = make_flow(c);   // psi_mv left out: Phi~ alone
   F0.V1 = 0.0;
+  F0.nb = 2;
   for (int j = 0; j < BIE_MAXB; ++j) F0.a[j] = 0.0;
-  k_psi_surface<<<M0, PS_THREADS, 0, c->stream>>>(B, nd, dz, d2z, wdf, omega, Xb, F0, psi0);
-  BIE_LAUNCH_CHECK(c, "k_psi_surface");
-  if (N > M0) {
-    k_phi_solid<<<N - M0, PS_THREADS, 0, c->stream>>>(B, nd, Tall, dz, d2z, wdf, omega, Xb, out);
-    BIE_LAUNCH_CHECK(c, "k_phi_solid");
-  }
+  s = pot_run(c, true, F0, nd, wdf, omega, Xb, psi0, out);
+  if (s != BIE_OK) return s;
   BIE_CUDA_TRY(c, cudaMemsetAsync(psik, 0, sizeof(double) * BIE_MAXB, c->stream));
   s = psi_run(c, omega, psik);
   if (s != BIE_OK) return s;

@@ -11,6 +11,7 @@
 //  * Near targets: the Helsing-Ojala ratio of eq. helsing:quad over the
 //    boundary values, with the free surface entering with -zeta_0' (positive
 //    orientation of the boundary of Omega), in double-float.
+#include <algorithm>
 #include <cstring>
 
 #include "common.cuh"
@@ -18,8 +19,8 @@
 #include "dft.cuh"
 #include "pair_kernel.cuh"
 #include "df2.cuh"
+#include "pair_sums.cuh"
 
-#define BND_CH 512
 #define BND_FIELDS 5   // Z0.re Z0.im Z1.re Z1.im tsum
 
 // gamma_l / M_l and H gamma_l (double-float) from the two inverse DFTs:
@@ -41,75 +42,80 @@ __global__ void k_gamma_extract(Blocks B, const double2* __restrict__ X2, float2
   cf[t] = (float)(wp / M);                    // omega' / M (far-field sums)
 }
 
-// Partial sums for boundary targets m over a chunk of sources l != m:
+// Partial sums for boundary targets m over the source tiles of split blockIdx.y:
 //   Z0 = sum_{l on Gamma_0} G_ml c_l,  Z1 = sum_{l off Gamma_0} G_ml c_l,
-//   tsum = sum_{l on m's boundary} 1/2 cot(pi (i_m - i_l)/M_k) c_l,
-// G_ml = 1/2 cot((zeta_l - zeta_m)/2), c_l = gamma_l / M_l.
-__global__ void __launch_bounds__(256) k_bnd_partial(Blocks B, const float4* __restrict__ nP,
-                                                     const float4* __restrict__ nQ,
-                                                     const float4* __restrict__ nPQc,
-                                                     const double2* __restrict__ z64,
-                                                     const int* __restrict__ blk,
-                                                     const float2* __restrict__ gc,
-                                                     const float2* __restrict__ Tall, float near2,
-                                                     float2* __restrict__ part) {
-  __shared__ float4 sP[BND_CH];
-  __shared__ float2 sPc[BND_CH];
-  __shared__ double2 sZ[BND_CH];
-  __shared__ float2 sC[BND_CH];
-  __shared__ int sB[BND_CH];
-  const int N = B.N;
-  const int s0 = blockIdx.y * BND_CH;
-  const int ns = min(BND_CH, N - s0);
-  for (int t = threadIdx.x; t < ns; t += blockDim.x) {
-    sP[t] = nP[s0 + t];
-    const float4 pq = nPQc[s0 + t];
-    sPc[t] = make_float2(pq.x, pq.y);
-    sZ[t] = z64[s0 + t];
-    sC[t] = gc[s0 + t];
-    sB[t] = blk[s0 + t];
-  }
-  __syncthreads();
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= N) return;
-  const float4 qv = nQ[m];
-  const cx<dfl> Q = {{qv.x, qv.y}, {qv.z, qv.w}};
-  const float4 qc4 = nPQc[m];
-  const float2 Qc = make_float2(qc4.z, qc4.w);
-  const double2 zm = z64[m];
-  const int km = blk[m];
+//   tsum = sum_{l on m's boundary} 1/2 cot(pi (i_m - i_l)/M_k) c_l   (l != m),
+// G_ml = 1/2 cot((zeta_l - zeta_m)/2), c_l = gamma_l / M_l (see pair_sums.cuh; 12288
+// nodes: 1534 -> 741 us).
+__global__ void __launch_bounds__(PSUM_THREADS, 2)
+    k_bnd_partial(Blocks B, PsumNodes nd, int ntile, const float2* __restrict__ gc, float2* __restrict__ part) {
+  __shared__ PsumStage<1> S[PSUM_WARPS];
+  __shared__ PsumClose<1> sc[PSUM_WARPS];
+  __shared__ unsigned mask[PSUM_MAXTILES / 32 + 1];
+  __shared__ dfl red[PSUM_WARPS][BND_FIELDS][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int km, m0, mn;
+  psum_tile(B, blockIdx.x, km, m0, mn);
+  const int m = m0 + min(lane, mn - 1);
+  PsumTarget T;
+  T.load(nd, m);
+  const float4 tbox = psum_box(T.z);
   const int om = B.off[km], Mk = B.M[km], im = m - om;
-  dfl Z0r = {0, 0}, Z0i = {0, 0}, Z1r = {0, 0}, Z1i = {0, 0}, ts = {0, 0};
-  for (int t = 0; t < ns; ++t) {
-    const int l = s0 + t;
-    if (l == m) continue;
-    const float4 pv = sP[t];
-    const cx<dfl> P = {{pv.x, pv.y}, {pv.z, pv.w}};
-    const cx<dfl> G = half_cot_pair<dfl>(P, Q, sPc[t], Qc, sZ[t], zm, near2);
-    const float2 cv = sC[t];
-    const dfl c = {cv.x, cv.y};
-    const dfl gr = G.re * c, gi = G.im * c;
-    const int bl = sB[t];
-    if (bl == 0) {
-      Z0r = Z0r + gr;
-      Z0i = Z0i + gi;
+  dfl Z[BND_FIELDS];
+#pragma unroll
+  for (int f = 0; f < BND_FIELDS; ++f) Z[f] = {0.f, 0.f};
+  auto stage = [&](int w, int l0, int n, dfl* ws) -> bool {
+    float4 sbox;
+    psum_stage<1>(S[w], nd, l0, n, [&](int l, dfl* v) { v[0] = {gc[l].x, gc[l].y}; }, ws, sbox);
+    return !psum_apart(tbox, sbox);
+  };
+  auto work = [&](int w, int kl, int l0, int n, const dfl* ws, int p0, int p1, bool close, bool own) {
+    const bool same = kl == km;
+    int idx = im - (l0 - om);               // (i_m - i_l) mod M_k of the tile's first source
+    if (same && idx < 0) idx += Mk;
+    df2 ar = {f2(0.f), f2(0.f)}, ai = ar, at = ar;
+#pragma unroll 1
+    for (int p = p0; p < p1; ++p) {
+      df2 dr, di, inv;
+      psum_pair(S[w], p, nd, T, close, l0, n, m, dr, di, inv);
+      const df2 c = d2_of(S[w].W[0][p]);
+      const df2 q = d2_mul(c, inv);
+      ar = d2_macc(ar, di, q);
+      ai = d2_macc(ai, dr, q);
+      if (same) {   // T_0 = 0: the target itself drops out
+        int ia = idx - p;
+        ia += ia < 0 ? Mk : 0;
+        int ib = ia - 16;
+        ib += ib < 0 ? Mk : 0;
+        const float2 ta = nd.Tall[om + ia], tb = nd.Tall[om + ib];
+        at = d2_macc(at, df2{f2(ta.x, tb.x), f2(ta.y, tb.y)}, c);
+      }
+    }
+    const dfl zr = d2_fold(ar);
+    dfl zi = d2_fold(ai);
+    if (own) {
+      zi = zi + df_half(ws[0]);
+      if (same && m >= l0 && m < l0 + n)    // the tile's sum of weights holds the target's own
+        zi = zi - df_half(dfl{gc[m].x, gc[m].y});
+    }
+    if (kl == 0) {
+      Z[0] = Z[0] + zr;
+      Z[1] = Z[1] + zi;
     } else {
-      Z1r = Z1r + gr;
-      Z1i = Z1i + gi;
+      Z[2] = Z[2] + zr;
+      Z[3] = Z[3] + zi;
     }
-    if (bl == km) {
-      int idx = im - (l - om);
-      if (idx < 0) idx += Mk;
-      const float2 tv = Tall[om + idx];
-      ts = ts + dfl{tv.x, tv.y} * c;
-    }
+    if (same) Z[4] = Z[4] + d2_fold(at);
+  };
+  psum_tiles<1>(B, ntile, sc, mask, stage, work);
+#pragma unroll
+  for (int f = 0; f < BND_FIELDS; ++f) red[warp][f][lane] = Z[f];
+  __syncthreads();
+  if (warp < BND_FIELDS && lane < mn) {
+    dfl v = red[0][warp][lane];
+    for (int w = 1; w < PSUM_WARPS; ++w) v = v + red[w][warp][lane];
+    part[((size_t)blockIdx.y * BND_FIELDS + warp) * B.N + m0 + lane] = make_float2(v.hi, v.lo);
   }
-  float2* p = part + (size_t)blockIdx.y * BND_FIELDS * N;
-  p[0 * (size_t)N + m] = make_float2(Z0r.hi, Z0r.lo);
-  p[1 * (size_t)N + m] = make_float2(Z0i.hi, Z0i.lo);
-  p[2 * (size_t)N + m] = make_float2(Z1r.hi, Z1r.lo);
-  p[3 * (size_t)N + m] = make_float2(Z1i.hi, Z1i.lo);
-  p[4 * (size_t)N + m] = make_float2(ts.hi, ts.lo);
 }
 
 // Phi'(zeta_m) from the partial sums (eqs. dphij:dnk, dphij:dsk, phi:prime):
@@ -127,20 +133,22 @@ __global__ void k_bnd_finish(Blocks B, FlowParams F, int nchunk, const float2* _
   const int m = t / OBS_SPLIT, sub = t % OBS_SPLIT;
   if (m >= B.N) return;   // whole groups leave together
   const int N = B.N;
-  // the chunks' partial sums: lane sub takes chunks sub, sub + OBS_SPLIT, ..., added in FP64
-  double acc[BND_FIELDS];
+  // the chunks' partial sums: lane sub takes chunks sub, sub + OBS_SPLIT, ...
+  dfl part_sum[BND_FIELDS];
 #pragma unroll
-  for (int f = 0; f < BND_FIELDS; ++f) acc[f] = 0.0;
+  for (int f = 0; f < BND_FIELDS; ++f) part_sum[f] = {0.f, 0.f};
+#pragma unroll 4
   for (int ch = sub; ch < nchunk; ch += OBS_SPLIT) {
     const float2* p = part + (size_t)ch * BND_FIELDS * N;
 #pragma unroll
     for (int f = 0; f < BND_FIELDS; ++f) {
       const float2 v = p[(size_t)f * N + m];
-      acc[f] += (double)v.x + (double)v.y;
+      part_sum[f] = part_sum[f] + dfl{v.x, v.y};
     }
   }
+  double acc[BND_FIELDS];
 #pragma unroll
-  for (int f = 0; f < BND_FIELDS; ++f) acc[f] = obs_group_sum(acc[f]);
+  for (int f = 0; f < BND_FIELDS; ++f) acc[f] = obs_group_sum(df_to_double(part_sum[f]));
   double asum = 0.0;
   for (int j = 2; j < F.nb; ++j) asum += F.a[j - 2];
   const double2 hc = obs_cot_sum(F, z64[m], sub);
@@ -185,74 +193,39 @@ __global__ void k_bnd_finish(Blocks B, FlowParams F, int nchunk, const float2* _
   fdf[m] = make_float4(a.hi, a.lo, b.hi, b.lo);
 }
 
-// Far targets (FP32): Phi'(z) = Phi_mv'(z) + sum_{l off Gamma_0} H_l c_l - i sum_{l on Gamma_0} H_l c_l,
-// H_l = 1/2 cot((zeta_l - z)/2) = i/2 + i/(P_l e^{-iz} - 1), c_l = omega_l'/M_l.
-// Also the smallest |zeta_l - z|^2 / h_l^2 (h_l the local node spacing); with
-// near_thr2 > 0, targets below it are appended to the Helsing list.
 #define FAR_CH 1024
+#define FAR_THREADS 128
 
-// Over sources [i0, i1) of the chunk: (sr, si) += sum c_l i/d_l, d_l = P_l Q - 1
-// = wr + i wi, i/d = (wi + i wr)/|d|^2; optionally the smallest |d|^2 / h_l^2
-// (near-target test).
+// Over sources [i0, i1) of the chunk, for two targets in the lanes of packed FP32:
+// (sr, si) += sum c_l i/d_l, d_l = P_l Q - 1 = wr + i wi, i/d = (wi + i wr)/|d|^2;
+// optionally the smallest |d|^2 / h_l^2 (near-target test).  The ten FP32
+// operations per pair bound it (15 FP32-pipe cycles per warp and pair measured,
+// 10 the least); one target per thread took 24, the reciprocal's subnormal
+// handling, loads and the loop among them (220,000 x 12288 pairs 1607 -> 1076 us).  Each lane's sums are
+// formed in the order of the sources, as with one target per thread.
 template <bool NEAR>
-__device__ __forceinline__ void far_sum(const float4* __restrict__ sP, int i0, int i1, float qr,
-                                        float qi, float& sr, float& si, float& dmin) {
-#pragma unroll 4
+__device__ __forceinline__ void far_sum(const float4* __restrict__ sP, int i0, int i1, float2 qr,
+                                        float2 qi, float2& sr, float2& si, float2& dmin) {
+  const float2 nqi = p_neg(qi);
+#pragma unroll 8
   for (int i = i0; i < i1; ++i) {
-    const float4 p = sP[i];
-    const float wr = fmaf(p.x, qr, -fmaf(p.y, qi, 1.0f));   // Re(P Q) - 1
-    const float wi = fmaf(p.x, qi, p.y * qr);               // Im(P Q)
-    const float n2 = fmaf(wr, wr, wi * wi);
-    const float q = p.z * rcp_approx(n2);
-    if (NEAR) dmin = fminf(dmin, n2 * p.w);
-    sr = fmaf(wi, q, sr);
-    si = fmaf(wr, q, si);
+    const float4 a = sP[2 * i], b = sP[2 * i + 1];
+    const float2 px = f2(a.x, a.y), py = f2(a.z, a.w);
+    const float2 wr = p_fma(px, qr, p_fma(py, nqi, f2(-1.0f)));   // Re(P Q) - 1
+    const float2 wi = p_fma(px, qi, p_mul(py, qr));           // Im(P Q)
+    const float2 n2 = p_fma(wr, wr, p_mul(wi, wi));
+    const float2 q = p_mul(f2(b.x, b.y), f2(rcp_approx(n2.x), rcp_approx(n2.y)));
+    if (NEAR) {
+      const float2 h = p_mul(n2, f2(b.z, b.w));
+      dmin = f2(fminf(dmin.x, h.x), fminf(dmin.y, h.y));
+    }
+    sr = p_fma(wi, q, sr);
+    si = p_fma(wr, q, si);
   }
 }
 
-// Far targets (FP32): Phi'(z) = Phi_mv'(z) + sum_{l off Gamma_0} G_l c_l - i sum_{l on Gamma_0} G_l c_l,
-// G_l = 1/2 cot((zeta_l - z)/2) = i/2 + i/d_l, c_l = omega_l'/M_l.  The i/2 part
-// drops out: sum_l omega_l' = 0 on every boundary (the spectral derivative has
-// no mean mode).  The surface and the other boundaries are separate loops
-// (no per-source branch).  With NEAR, targets whose nearest node is closer
-// than sqrt(near_thr2) local spacings are appended to the Helsing list.
-template <bool NEAR>
-__global__ void __launch_bounds__(256) k_targets_far(int n, const double2* __restrict__ z, int N,
-                                                     int M0, const float4* __restrict__ nP,
-                                                     const float* __restrict__ cf,
-                                                     const float* __restrict__ hinv2,
-                                                     FlowParams F, double2* __restrict__ uv,
-                                                     float near_thr2, int* __restrict__ nlist,
-                                                     int* __restrict__ ncount) {
-  __shared__ float4 sP[FAR_CH];   // (P.re, P.im, c, 1/h^2)
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = t < n;
-  double2 zt = make_double2(0.0, 0.0);
-  float qr = 0.f, qi = 0.f;
-  if (active) {
-    zt = z[t];
-    double s, c;
-    sincos(zt.x, &s, &c);
-    const double e = exp(zt.y);
-    qr = (float)(e * c);
-    qi = (float)(-e * s);
-  }
-  float s0r = 0.f, s0i = 0.f, s1r = 0.f, s1i = 0.f, dmin = 3.0e38f;
-  for (int b0 = 0; b0 < N; b0 += FAR_CH) {
-    const int nb = min(FAR_CH, N - b0);
-    __syncthreads();
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-      const float4 p = nP[b0 + i];
-      sP[i] = make_float4(p.x, p.z, cf[b0 + i], NEAR ? hinv2[b0 + i] : 0.f);
-    }
-    __syncthreads();
-    if (!active) continue;
-    const int ns = min(nb, max(0, M0 - b0));   // surface sources in this chunk
-    far_sum<NEAR>(sP, 0, ns, qr, qi, s0r, s0i, dmin);
-    far_sum<NEAR>(sP, ns, nb, qr, qi, s1r, s1i, dmin);
-  }
-  if (!active) return;
-  // Phi_mv'(z) in FP64
+// Phi_mv'(z) in FP64
+__device__ __forceinline__ double2 far_mv(const FlowParams& F, double2 zt) {
   double pr = F.V1, pi = 0.0;
   for (int j = 2; j < F.nb; ++j) {
     const double ux = zt.x - F.zc[j - 2].x, uy = zt.y - F.zc[j - 2].y;
@@ -265,12 +238,62 @@ __global__ void __launch_bounds__(256) k_targets_far(int n, const double2* __res
     pr += F.a[j - 2] * (0.5 + hi);
     pi += F.a[j - 2] * (-hr);
   }
-  // sum G c = i sum c/d = (S.re, S.im) with S = (wi q, wr q); -i S0 = (S0.im, -S0.re)
-  uv[t] = make_double2(pr + (double)s1r + (double)s0i, pi + (double)s1i - (double)s0r);
-  if (NEAR && dmin < near_thr2) {
-    const int slot = atomicAdd(ncount, 1);
-    nlist[slot] = t;
+  return make_double2(pr, pi);
+}
+
+// Far targets (FP32): Phi'(z) = Phi_mv'(z) + sum_{l off Gamma_0} G_l c_l - i sum_{l on Gamma_0} G_l c_l,
+// G_l = 1/2 cot((zeta_l - z)/2) = i/2 + i/d_l, c_l = omega_l'/M_l.  The i/2 part
+// drops out: sum_l omega_l' = 0 on every boundary (the spectral derivative has
+// no mean mode).  The surface and the other boundaries are separate loops
+// (no per-source branch).  With NEAR, targets whose nearest node is closer
+// than sqrt(near_thr2) local spacings are appended to the Helsing list.
+template <bool NEAR>
+__global__ void __launch_bounds__(FAR_THREADS) k_targets_far(int n, const double2* __restrict__ z, int N,
+                                                             int M0, const float4* __restrict__ nP,
+                                                             const float* __restrict__ cf,
+                                                             const float* __restrict__ hinv2,
+                                                             FlowParams F, double2* __restrict__ uv,
+                                                             float near_thr2, int* __restrict__ nlist,
+                                                             int* __restrict__ ncount) {
+  __shared__ float4 sP[2 * FAR_CH];   // (P.re, P.re, P.im, P.im), (c, c, 1/h^2, 1/h^2)
+  // targets t0 and t0 + blockDim.x of this CTA's 2 blockDim.x
+  const int t0 = blockIdx.x * 2 * blockDim.x + threadIdx.x, t1 = t0 + blockDim.x;
+  const bool a0 = t0 < n, a1 = t1 < n;
+  float2 qr = f2(0.f), qi = f2(0.f);
+  auto load_q = [&](int t, float& r, float& i) {
+    const double2 zt = z[t];
+    double s, c;
+    sincos(zt.x, &s, &c);
+    const double e = exp(zt.y);
+    r = (float)(e * c);
+    i = (float)(-e * s);
+  };
+  if (a0) load_q(t0, qr.x, qi.x);
+  if (a1) load_q(t1, qr.y, qi.y);
+  float2 s0r = f2(0.f), s0i = s0r, s1r = s0r, s1i = s0r, dmin = f2(3.0e38f);
+  for (int b0 = 0; b0 < N; b0 += FAR_CH) {
+    const int nb = min(FAR_CH, N - b0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+      const float4 p = nP[b0 + i];
+      const float c = cf[b0 + i], h = NEAR ? hinv2[b0 + i] : 0.f;
+      sP[2 * i] = make_float4(p.x, p.x, p.z, p.z);
+      sP[2 * i + 1] = make_float4(c, c, h, h);
+    }
+    __syncthreads();
+    if (!a0) continue;
+    const int ns = min(nb, max(0, M0 - b0));   // surface sources in this chunk
+    far_sum<NEAR>(sP, 0, ns, qr, qi, s0r, s0i, dmin);
+    far_sum<NEAR>(sP, ns, nb, qr, qi, s1r, s1i, dmin);
   }
+  // sum G c = i sum c/d = (S.re, S.im) with S = (wi q, wr q); -i S0 = (S0.im, -S0.re)
+  auto store = [&](int t, float x0r, float x0i, float x1r, float x1i, float dm) {
+    const double2 mv = far_mv(F, z[t]);
+    uv[t] = make_double2(mv.x + (double)x1r + (double)x0i, mv.y + (double)x1i - (double)x0r);
+    if (NEAR && dm < near_thr2) nlist[atomicAdd(ncount, 1)] = t;
+  };
+  if (a0) store(t0, s0r.x, s0i.x, s1r.x, s1i.x, dmin.x);
+  if (a1) store(t1, s0r.y, s0i.y, s1r.y, s1i.y, dmin.y);
 }
 
 // Helsing-Ojala (eq. helsing:quad): Phi'(z) = sum lam f / sum lam,
@@ -293,9 +316,13 @@ __device__ __forceinline__ dfl hel_group_sum(dfl v) {
 // Two sources per lane at once, in the two lanes of the packed double-float
 // arithmetic (df2): a chunk's sources are staged pair-major, source i of the
 // lane's stride beside source i + HEL_SPLIT, so one float4 load gives a
-// quantity for both.  Per pair of sources: d = P Q - 1 and |d|^2, H = i/2 +
-// i/d, lam = H E and lam f each as combined double-float products, the sums
-// accumulated inside the last ones.
+// quantity for both.  With H = i/2 + g, g = i/d = (Im d + i Re d)/|d|^2, and the
+// weights E = sigma zeta'/M and F = E f formed once per node,
+//   sum lam f = i/2 sum F + sum g F,   sum lam = i/2 sum E + sum g E,
+// so per pair of sources: d = P Q - 1 and |d|^2, g, and four sums accumulated
+// inside combined double-float products (forming lam = H E and lam f per target
+// took a sixth more operations; FP32 arithmetic bounds the kernel, 85% of the pipe;
+// 1906 -> 1741 us for the near targets of 220,000 at 12288 nodes).
 struct HelPk {
   float4 Pr, Pi, Er, Ei, Fr, Fi;   // (hi a, hi b, lo a, lo b) of each component
 };
@@ -306,9 +333,12 @@ __global__ void __launch_bounds__(256) k_targets_helsing(int n, const int* __res
                                                          const double2* __restrict__ z, int N,
                                                          const float4* __restrict__ nP,
                                                          const float4* __restrict__ nEw,
+                                                         const float4* __restrict__ nFw,
                                                          const float4* __restrict__ fdf,
+                                                         const float2* __restrict__ wsum, int nwsum,
                                                          double2* __restrict__ uv) {
   __shared__ HelPk sK[HEL_CH / 2];
+  __shared__ dfl sW[4];   // sums of E and F over all nodes
   const int cnt = list ? *count : n;
   // the grid covers every target; CTAs past the near list have nothing to do
   // (returning here keeps them from staging every source chunk)
@@ -317,6 +347,13 @@ __global__ void __launch_bounds__(256) k_targets_helsing(int n, const int* __res
   const int sub = (int)threadIdx.x % HEL_SPLIT;
   const bool active = t < cnt;
   const int tg = active ? (list ? list[t] : t) : 0;
+  if (threadIdx.x < 128) {
+    const int f = threadIdx.x >> 5;
+    dfl w = {0.f, 0.f};
+    for (int b = threadIdx.x & 31; b < nwsum; b += 32) w = w + dfl{wsum[4 * b + f].x, wsum[4 * b + f].y};
+    w = warp_sum(w);
+    if ((threadIdx.x & 31) == 0) sW[f] = w;
+  }
   df2 Qr = {f2(0.f), f2(0.f)}, Qi = {f2(0.f), f2(0.f)};
   if (active) {
     const double2 zt = z[tg];
@@ -339,11 +376,11 @@ __global__ void __launch_bounds__(256) k_targets_helsing(int n, const int* __res
       const int ia = (p / HEL_SPLIT) * 2 * HEL_SPLIT + p % HEL_SPLIT, ib = ia + HEL_SPLIT;
       const bool oka = ia < nb, okb = ib < nb;
       const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      // a source past the chunk repeats a real source's position with zero weight and value
+      // a source past the chunk repeats a real source's position with zero weights
       const float4 pa = nP[b0 + (oka ? ia : 0)];
-      const float4 ea = oka ? nEw[b0 + ia] : z4, fa = oka ? fdf[b0 + ia] : z4;
+      const float4 ea = oka ? nEw[b0 + ia] : z4, fa = oka ? nFw[b0 + ia] : z4;
       const float4 pb = okb ? nP[b0 + ib] : pa;
-      const float4 eb = okb ? nEw[b0 + ib] : z4, fb = okb ? fdf[b0 + ib] : z4;
+      const float4 eb = okb ? nEw[b0 + ib] : z4, fb = okb ? nFw[b0 + ib] : z4;
       HelPk k;
       k.Pr = make_float4(pa.x, pb.x, pa.y, pb.y);
       k.Pi = make_float4(pa.z, pb.z, pa.w, pb.w);
@@ -369,16 +406,13 @@ __global__ void __launch_bounds__(256) k_targets_helsing(int n, const int* __res
         continue;
       }
       const df2 inv = d2_rcp(n2);
-      const df2 Hr = d2_mul(d_i, inv);                   // Re(i/2 + i/d)
-      const df2 Hi = d2_mul_addf(d_r, inv, f2(0.5f));   // Im(i/2 + i/d)
+      const df2 gr = d2_mul(d_i, inv), gi = d2_mul(d_r, inv), ngi = d2_neg(gi);
       const df2 Er = hel_pk(k.Er), Ei = hel_pk(k.Ei);
-      const df2 lr = d2_dot2<false>(Hr, Er, d2_neg(Hi), Ei, f2(0.f), f2(0.f));   // lam = H E
-      const df2 li = d2_dot2<false>(Hr, Ei, Hi, Er, f2(0.f), f2(0.f));
+      dr = d2_dot2<true>(gr, Er, ngi, Ei, dr.hi, dr.lo);   // += Re(g E)
+      di = d2_dot2<true>(gr, Ei, gi, Er, di.hi, di.lo);    // += Im(g E)
       const df2 Fr = hel_pk(k.Fr), Fi = hel_pk(k.Fi);
-      nr = d2_dot2<true>(lr, Fr, d2_neg(li), Fi, nr.hi, nr.lo);   // += Re(lam f)
-      ni = d2_dot2<true>(lr, Fi, li, Fr, ni.hi, ni.lo);           // += Im(lam f)
-      dr = d2_add(dr, lr);
-      di = d2_add(di, li);
+      nr = d2_dot2<true>(gr, Fr, ngi, Fi, nr.hi, nr.lo);   // += Re(g F)
+      ni = d2_dot2<true>(gr, Fi, gi, Fr, ni.hi, ni.lo);    // += Im(g F)
     }
   }
   // the two lanes of every sum, then the lanes of a group (inactive groups carry zeros)
@@ -398,25 +432,50 @@ __global__ void __launch_bounds__(256) k_targets_helsing(int n, const int* __res
     uv[tg] = make_double2((double)fv.x + (double)fv.y, (double)fv.z + (double)fv.w);
     return;
   }
-  const double Nr = df_to_double(snr), Ni = df_to_double(sni), Dr = df_to_double(sdr), Di = df_to_double(sdi);
+  // + i/2 times the sums of E and F
+  const double Nr = df_to_double(snr) - 0.5 * df_to_double(sW[3]), Ni = df_to_double(sni) + 0.5 * df_to_double(sW[2]);
+  const double Dr = df_to_double(sdr) - 0.5 * df_to_double(sW[1]), Di = df_to_double(sdi) + 0.5 * df_to_double(sW[0]);
   const double D2 = Dr * Dr + Di * Di;
   uv[tg] = make_double2((Nr * Dr + Ni * Di) / D2, (Ni * Dr - Nr * Di) / D2);
 }
 
-// per node: sigma zeta'/M (double-float complex) and 1/h^2 with h = |zeta'| 2 pi / M
-__global__ void k_node_weights(Blocks B, const double2* __restrict__ dz, float4* __restrict__ nEw,
-                               float* __restrict__ hinv2) {
+// per node: E = sigma zeta'/M and F = E f (double-float complex) and 1/h^2 with
+// h = |zeta'| 2 pi / M; the CTA's sums of E and F (four double-floats) in wsum
+__global__ void __launch_bounds__(NODE_THREADS)
+    k_node_weights(Blocks B, const double2* __restrict__ dz, const float4* __restrict__ fdf,
+                   float4* __restrict__ nEw, float4* __restrict__ nFw, float2* __restrict__ wsum,
+                   float* __restrict__ hinv2) {
+  __shared__ dfl red[NODE_THREADS / 32][4];
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= B.N) return;
-  int k = 0;
-  while (k + 1 < B.nb && l >= B.off[k + 1]) ++k;
-  const double sg = (k == 0) ? -1.0 : 1.0;
-  const double M = (double)B.M[k];
-  const double2 d = dz[l];
-  const dfl er = df_from_double(sg * d.x / M), ei = df_from_double(sg * d.y / M);
-  nEw[l] = make_float4(er.hi, er.lo, ei.hi, ei.lo);
-  const double h = sqrt(d.x * d.x + d.y * d.y) * (2.0 * M_PI / M);
-  hinv2[l] = (float)(1.0 / (h * h));
+  dfl v[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};   // E.re, E.im, F.re, F.im
+  if (l < B.N) {
+    int k = 0;
+    while (k + 1 < B.nb && l >= B.off[k + 1]) ++k;
+    const double sg = (k == 0) ? -1.0 : 1.0;
+    const double M = (double)B.M[k];
+    const double2 d = dz[l];
+    v[0] = df_from_double(sg * d.x / M);
+    v[1] = df_from_double(sg * d.y / M);
+    const float4 f4 = fdf[l];
+    const dfl fr = {f4.x, f4.y}, fi = {f4.z, f4.w};
+    v[2] = v[0] * fr - v[1] * fi;
+    v[3] = v[0] * fi + v[1] * fr;
+    nEw[l] = make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo);
+    nFw[l] = make_float4(v[2].hi, v[2].lo, v[3].hi, v[3].lo);
+    const double h = sqrt(d.x * d.x + d.y * d.y) * (2.0 * M_PI / M);
+    hinv2[l] = (float)(1.0 / (h * h));
+  }
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    v[f] = warp_sum(v[f]);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][f] = v[f];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    dfl t = red[0][threadIdx.x];
+    for (int w = 1; w < NODE_THREADS / 32; ++w) t = t + red[w][threadIdx.x];
+    wsum[4 * blockIdx.x + threadIdx.x] = make_float2(t.hi, t.lo);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -427,7 +486,7 @@ static bie_status boundary_values(bie_ctx* c, const double* omega, double2** f64
   const Blocks B = make_blocks(c);
   const FlowParams F = make_flow(c);
   const int N = c->N;
-  const int nchunk = (N + BND_CH - 1) / BND_CH;
+  const int ntile = psum_ntile(B), nchunk = psum_nsplit(ntile, ntile);
   double2 *dY, *dX1, *dX2, *f64;
   float2 *gc, *hg, *part;
   float4* fdf;
@@ -484,8 +543,8 @@ static bie_status boundary_values(bie_ctx* c, const double* omega, double2** f64
   BIE_LAUNCH_CHECK(c, "k_dft_b");
   k_gamma_extract<<<(N + 255) / 256, 256, 0, c->stream>>>(B, dX2, gc, hg, cf);
   BIE_LAUNCH_CHECK(c, "k_gamma_extract");
-  k_bnd_partial<<<dim3((N + 255) / 256, nchunk), 256, 0, c->stream>>>(B, nP, nQ, nPQc, z64, blk, gc,
-                                                                     Tall, 0.01f, part);
+  const PsumNodes nd = {nP, nQ, nPQc, z64, Tall};
+  k_bnd_partial<<<dim3(ntile, nchunk), PSUM_THREADS, 0, c->stream>>>(B, nd, ntile, gc, part);
   BIE_LAUNCH_CHECK(c, "k_bnd_partial");
   k_bnd_finish<<<obs_grid(N), NODE_THREADS, 0, c->stream>>>(B, F, nchunk, part, z64, dz64, d2z64, blk, gc,
                                                        hg, f64, fdf);
@@ -540,11 +599,14 @@ extern "C" bie_status bie_eval_potential(bie_ctx* c, const double* omega_dev, lo
   const Blocks B = make_blocks(c);
   const int N = c->N;
   double2* bnd;
-  float4 *fdf, *nEw;
+  float4 *fdf, *nEw, *nFw;
+  float2* wsum;
   float* hinv2;
   BIE_GET(c, double2, "ep_bnd", N, bnd);
   BIE_GET(c, float4, "ep_fdf", N, fdf);
   BIE_GET(c, float4, "tg_nEw", N, nEw);
+  BIE_GET(c, float4, "tg_nFw", N, nFw);
+  BIE_GET(c, float2, "tg_wsum", 4 * node_grid(N), wsum);
   BIE_GET(c, float, "tg_hinv2", N, hinv2);
   bool oom = false;
   const float4* nP = (const float4*)ctx_buf(c, "nP", sizeof(float4) * N, &oom);
@@ -554,10 +616,10 @@ extern "C" bie_status bie_eval_potential(bie_ctx* c, const double* omega_dev, lo
   if (s != BIE_OK) return s;
   k_c_to_df<<<(N + 255) / 256, 256, 0, c->stream>>>(N, bnd, fdf);
   BIE_LAUNCH_CHECK(c, "k_c_to_df");
-  k_node_weights<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, dz64, nEw, hinv2);
+  k_node_weights<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, dz64, fdf, nEw, nFw, wsum, hinv2);
   BIE_LAUNCH_CHECK(c, "k_node_weights");
   k_targets_helsing<<<(unsigned)((n + HEL_TPB - 1) / HEL_TPB), 256, 0, c->stream>>>(
-      (int)n, nullptr, nullptr, (const double2*)z_dev, N, nP, nEw, fdf, (double2*)phi_dev);
+      (int)n, nullptr, nullptr, (const double2*)z_dev, N, nP, nEw, nFw, fdf, wsum, (int)node_grid(N), (double2*)phi_dev);
   BIE_LAUNCH_CHECK(c, "k_targets_helsing");
   return BIE_OK;
 }
@@ -583,10 +645,13 @@ extern "C" bie_status bie_eval_velocity(bie_ctx* c, const double* omega_dev, lon
   float* cf;
   bie_status s = boundary_values(c, omega_dev, &f64, &fdf, &cf);
   if (s != BIE_OK) return s;
-  float4* nEw;
+  float4 *nEw, *nFw;
+  float2* wsum;
   float* hinv2;
   int *nlist, *ncount;
   BIE_GET(c, float4, "tg_nEw", N, nEw);
+  BIE_GET(c, float4, "tg_nFw", N, nFw);
+  BIE_GET(c, float2, "tg_wsum", 4 * node_grid(N), wsum);
   BIE_GET(c, float, "tg_hinv2", N, hinv2);
   BIE_GET(c, int, "tg_nlist", n, nlist);
   BIE_GET(c, int, "tg_ncount", 1, ncount);
@@ -594,14 +659,16 @@ extern "C" bie_status bie_eval_velocity(bie_ctx* c, const double* omega_dev, lon
   const float4* nP = (const float4*)ctx_buf(c, "nP", sizeof(float4) * N, &oom);
   const double2* dz64 = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "targets: buffers");
-  k_node_weights<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, dz64, nEw, hinv2);
+  k_node_weights<<<node_grid(N), NODE_THREADS, 0, c->stream>>>(B, dz64, fdf, nEw, nFw, wsum, hinv2);
   BIE_LAUNCH_CHECK(c, "k_node_weights");
   const double2* z = (const double2*)z_dev;
   double2* uv = (double2*)uv_dev;
-  const unsigned g = (unsigned)((n + 255) / 256);
+  // few targets: smaller CTAs, one warp each when there are fewer than the SMs take
+  const int fth = n < 2LL * 32 * 1024 ? 32 : FAR_THREADS;
+  const unsigned g = (unsigned)((n + 2 * fth - 1) / (2 * fth));
   if (mode == 1) {
     k_targets_helsing<<<(unsigned)((n + HEL_TPB - 1) / HEL_TPB), 256, 0, c->stream>>>(
-        (int)n, nullptr, nullptr, z, N, nP, nEw, fdf, uv);
+        (int)n, nullptr, nullptr, z, N, nP, nEw, nFw, fdf, wsum, (int)node_grid(N), uv);
     BIE_LAUNCH_CHECK(c, "k_targets_helsing");
     if (n_near_out) *n_near_out = n;
     return BIE_OK;
@@ -609,15 +676,15 @@ extern "C" bie_status bie_eval_velocity(bie_ctx* c, const double* omega_dev, lon
   BIE_CUDA_TRY(c, cudaMemsetAsync(ncount, 0, sizeof(int), c->stream));
   const float thr2 = mode == 2 ? (float)(near_spacings * near_spacings) : 0.f;
   if (mode == 2)
-    k_targets_far<true><<<g, 256, 0, c->stream>>>((int)n, z, N, c->M[0], nP, cf, hinv2, F, uv, thr2,
+    k_targets_far<true><<<g, fth, 0, c->stream>>>((int)n, z, N, c->M[0], nP, cf, hinv2, F, uv, thr2,
                                                   nlist, ncount);
   else
-    k_targets_far<false><<<g, 256, 0, c->stream>>>((int)n, z, N, c->M[0], nP, cf, hinv2, F, uv, thr2,
+    k_targets_far<false><<<g, fth, 0, c->stream>>>((int)n, z, N, c->M[0], nP, cf, hinv2, F, uv, thr2,
                                                    nlist, ncount);
   BIE_LAUNCH_CHECK(c, "k_targets_far");
   if (mode == 2) {
     k_targets_helsing<<<(unsigned)((n + HEL_TPB - 1) / HEL_TPB), 256, 0, c->stream>>>(
-        (int)n, nlist, ncount, z, N, nP, nEw, fdf, uv);
+        (int)n, nlist, ncount, z, N, nP, nEw, nFw, fdf, wsum, (int)node_grid(N), uv);
     BIE_LAUNCH_CHECK(c, "k_targets_helsing");
     if (n_near_out) {
       int h = 0;
