@@ -549,16 +549,6 @@ __global__ void __launch_bounds__(256) k_adj_shape(Blocks B, EllParams E,
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-static bie_status dft_pass(bie_ctx* c, const DftJobs& J, const double* xr, const double2* xc,
-                           const double2* tw, double2* Y, double2* X) {
-  const unsigned g = (unsigned)((J.total + 255) / 256);
-  k_dft_a<<<dft_grid(g), 256, 0, c->stream>>>(J, xr, xc, tw, Y);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(g), 256, 0, c->stream>>>(J, Y, tw, X);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  return BIE_OK;
-}
-
 // D applied to a complex vector on every boundary: X2 = DFT(conj(i k DFT(x)))
 static bie_status spectral_d(bie_ctx* c, const double2* x, const double2* tw, double2* Y,
                              double2* X1, double2* X2) {
@@ -573,9 +563,9 @@ static bie_status spectral_d(bie_ctx* c, const double2* x, const double2* tw, do
     s += M;
   }
   J1.total = J2.total = s;
-  bie_status st = dft_pass(c, J1, nullptr, x, tw, Y, X1);
+  bie_status st = dft_run(c, J1, nullptr, x, Y, X1);
   if (st != BIE_OK) return st;
-  return dft_pass(c, J2, nullptr, X1, tw, Y, X2);
+  return dft_run(c, J2, nullptr, X1, Y, X2);
 }
 
 extern "C" bie_status bie_backward(bie_ctx* c, const double* omega, const double* gU,
@@ -723,9 +713,9 @@ extern "C" bie_status bie_backward(bie_ctx* c, const double* omega, const double
       t += M;
     }
     J1.total = J2.total = t;
-    s = dft_pass(c, J1, xin, nullptr, tw, dY, dX1);
+    s = dft_run(c, J1, xin, nullptr, dY, dX1);
     if (s != BIE_OK) return s;
-    s = dft_pass(c, J2, nullptr, dX1, tw, dY, dX2);
+    s = dft_run(c, J2, nullptr, dX1, dY, dX2);
     if (s != BIE_OK) return s;
   }
   k_adj_rhs<<<(N + 255) / 256, 256, 0, c->stream>>>(B, dX2, omega, nbar, rhs, coef);

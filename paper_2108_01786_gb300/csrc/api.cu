@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "nvtx.cuh"
+#include "dft.cuh"
 
 // ---------------------------------------------------------------------------
 // context helpers
@@ -483,6 +484,8 @@ bie_status geometry_prep(bie_ctx* c) {
     c->spec_nb = 0;
     k_spectral_tables<<<(c->N + nthr - 1) / nthr, nthr, 0, c->stream>>>(B, tw, Ttab, T64, Tall);
     BIE_LAUNCH_CHECK(c, "k_spectral_tables");
+    const bie_status sd = dft_tables(c);
+    if (sd != BIE_OK) return sd;
     for (int k = 0; k < c->nb; ++k) c->spec_M[k] = c->M[k];
     c->spec_nb = c->nb;
   }

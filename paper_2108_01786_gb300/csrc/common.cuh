@@ -205,7 +205,7 @@ struct bie_ctx {
   int M[BIE_MAXB] = {0};
   int off[BIE_MAXB + 1] = {0};
   double2 zc[BIE_MAXB] = {};
-  int fft_m1[BIE_MAXB] = {0};   // four-step DFT factor M1 of each boundary (M = M1 M2)
+  int fft_m1[BIE_MAXB] = {0};   // DFT factor M1 of each boundary (M = M1 M2)
   bool have_geom = false;
   bool have_flow = false;
   double V1 = 0.0;
@@ -249,6 +249,9 @@ struct bie_ctx {
   // node counts the spectral tables (twiddles, cotangent tables) were built for
   int spec_M[BIE_MAXB] = {};
   int spec_nb = 0;
+  // Bluestein transforms (dft.cu): padded length per boundary (0: not taken), table offsets
+  int bl_q[BIE_MAXB] = {0};
+  int bl_off[BIE_MAXB] = {0};
 
   // pinned status mirror, host-mapped step ring and its events
   SolveStatus* status_host = nullptr;

@@ -57,7 +57,6 @@ bie_status graph_derivs(bie_ctx* c, const double* y, double2* X2) {
   BIE_GET(c, double2, "ev_Y", 3 * (size_t)M0, dY);
   BIE_GET(c, double2, "ev_X1", 2 * (size_t)M0, dX1);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * c->N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "evolve: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
@@ -69,14 +68,8 @@ bie_status graph_derivs(bie_ctx* c, const double* y, double2* X2) {
   J2.j[J2.n++] = DftJob{M0, M1, M2, M0, M0, 0, 1, M0};
   J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 2 * M0, 0, 5, 2 * M0};
   J2.total = 3 * M0;
-  k_dft_a<<<dft_grid((J1.total + 255) / 256), 256, 0, c->stream>>>(J1, y, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid((J1.total + 255) / 256), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid((J2.total + 255) / 256), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid((J2.total + 255) / 256), 256, 0, c->stream>>>(J2, dY, tw, X2);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, y, nullptr, dY, dX1)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, X2)) return sd;
   return BIE_OK;
 }
 
@@ -413,7 +406,6 @@ bie_status energy_run(bie_ctx* c, const double* phit, const double* omega, doubl
   BIE_GET(c, double, "en_psi0", M0, psi0);
   BIE_GET(c, double, "en_psik", BIE_MAXB, psik);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   const double2* z = (const double2*)ctx_buf(c, "zeta", sizeof(double2) * N, &oom);
   const double2* dz = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
   const double2* d2z = (const double2*)ctx_buf(c, "d2zeta", sizeof(double2) * N, &oom);
@@ -427,32 +419,16 @@ bie_status energy_run(bie_ctx* c, const double* phit, const double* omega, doubl
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "energy: buffers");
   // H omega_0 (mode 4) at [0, M0) and phi~_alpha (mode 1) at [M0, 2 M0):
   // forward passes of omega_0 and phi~ into X1, inverse passes into X2
-  DftJobs Jw, Jp, Jb, J2;
-  memset(&Jw, 0, sizeof(Jw));
-  memset(&Jp, 0, sizeof(Jp));
-  memset(&Jb, 0, sizeof(Jb));
+  DftJobs J1, J2;
+  memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  Jw.j[Jw.n++] = DftJob{M0, M1, M2, 0, 0, 0, 0, 0};
-  Jw.total = M0;
-  Jp.j[Jp.n++] = DftJob{M0, M1, M2, 0, M0, 0, 0, 0};
-  Jp.total = M0;
-  Jb.j[Jb.n++] = DftJob{M0, M1, M2, 0, 0, 0, 0, 0};
-  Jb.j[Jb.n++] = DftJob{M0, M1, M2, M0, M0, 0, 0, M0};
-  Jb.total = 2 * M0;
+  J1.j[J1.n++] = DftJob{M0, M1, M2, 0, 0, 0, 0, 0};
+  J1.j[J1.n++] = DftJob{M0, M1, M2, 0, M0, 0, 8, M0};
   J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 0, 0, 4, 0};
   J2.j[J2.n++] = DftJob{M0, M1, M2, M0, M0, 0, 1, M0};
-  J2.total = 2 * M0;
-  const unsigned g1 = (unsigned)((M0 + 255) / 256), g2 = (unsigned)((2 * M0 + 255) / 256);
-  k_dft_a<<<dft_grid(g1), 256, 0, c->stream>>>(Jw, omega, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_a<<<dft_grid(g1), 256, 0, c->stream>>>(Jp, phit, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(g2), 256, 0, c->stream>>>(Jb, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid(g2), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(g2), 256, 0, c->stream>>>(J2, dY, tw, dX2);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  J1.total = J2.total = 2 * M0;
+  if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX1, 1, 0, 0, phit)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   const Blocks B = make_blocks(c);
   const FlowParams F = make_flow(c);
   float2* wdf;
@@ -493,7 +469,6 @@ bie_status filter_run(bie_ctx* c, double* x, int nv) {
   BIE_GET(c, double2, "fl_Y", 2 * (size_t)M0, dY);
   BIE_GET(c, double2, "fl_X1", 2 * (size_t)M0, dX1);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * c->N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "filter: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
@@ -504,14 +479,8 @@ bie_status filter_run(bie_ctx* c, double* x, int nv) {
   }
   J1.total = J2.total = nv * M0;
   const unsigned gb = (unsigned)((nv * M0 + 255) / 256);
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J1, x, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J2, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, x, nullptr, dY, dX1)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX1)) return sd;
   k_take_real_mode<<<gb, 256, 0, c->stream>>>(nv * M0, M0, dX1, x);
   BIE_LAUNCH_CHECK(c, "k_take_real_mode");
   return BIE_OK;
@@ -525,7 +494,6 @@ bie_status dft_pair(bie_ctx* c, const double* x, int m0, int m1, double2* out) {
   BIE_GET(c, double2, "hp_Y", 2 * (size_t)M0, dY);
   BIE_GET(c, double2, "hp_X1", 2 * (size_t)M0, dX1);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * c->N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "dft: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
@@ -535,15 +503,8 @@ bie_status dft_pair(bie_ctx* c, const double* x, int m0, int m1, double2* out) {
   J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 0, 0, m0, 0};
   J2.j[J2.n++] = DftJob{M0, M1, M2, M0, M0, 0, m1, M0};
   J1.total = J2.total = 2 * M0;
-  const unsigned gb = (unsigned)((2 * M0 + 255) / 256);
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J1, x, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J2, dY, tw, out);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, x, nullptr, dY, dX1)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, out)) return sd;
   return BIE_OK;
 }
 
@@ -774,7 +735,6 @@ bie_status dft_blocks(bie_ctx* c, const double* x, int mode, double2* out) {
   BIE_GET(c, double2, "db_Y", N, dY);
   BIE_GET(c, double2, "db_X1", N, dX1);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "dft: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
@@ -785,15 +745,8 @@ bie_status dft_blocks(bie_ctx* c, const double* x, int mode, double2* out) {
     J2.j[J2.n++] = DftJob{M, M1, M / M1, o, o, o, mode, o};
   }
   J1.total = J2.total = N;
-  const unsigned gb = (unsigned)((N + 255) / 256);
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J1, x, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J2, dY, tw, out);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, x, nullptr, dY, dX1)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, out)) return sd;
   return BIE_OK;
 }
 

@@ -501,7 +501,6 @@ static bie_status boundary_values(bie_ctx* c, const double* omega, double2** f64
   BIE_GET(c, double2, "tg_f64", N, f64);
   BIE_GET(c, float4, "tg_fdf", N, fdf);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   const float2* Tall = (const float2*)ctx_buf(c, "Tall", sizeof(float2) * N, &oom);
   const float4* nP = (const float4*)ctx_buf(c, "nP", sizeof(float4) * N, &oom);
   const float4* nQ = (const float4*)ctx_buf(c, "nQ", sizeof(float4) * N, &oom);
@@ -533,14 +532,8 @@ static bie_status boundary_values(bie_ctx* c, const double* omega, double2** f64
   }
   J1.total = s1;
   J2.total = s2;
-  k_dft_a<<<dft_grid((s1 + 255) / 256), 256, 0, c->stream>>>(J1, omega, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid((s1 + 255) / 256), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid((s2 + 255) / 256), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid((s2 + 255) / 256), 256, 0, c->stream>>>(J2, dY, tw, dX2);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX1)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   k_gamma_extract<<<(N + 255) / 256, 256, 0, c->stream>>>(B, dX2, gc, hg, cf);
   BIE_LAUNCH_CHECK(c, "k_gamma_extract");
   const PsumNodes nd = {nP, nQ, nPQc, z64, Tall};

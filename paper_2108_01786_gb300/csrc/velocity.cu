@@ -50,130 +50,6 @@ __device__ __forceinline__ cx<dfl> near_R_v(double2 zl, double2 zm) {
   return c_mul(D, E);
 }
 
-// ---------------------------------------------------------------------------
-// Spectral derivative and Hilbert transform by a four-step DFT in FP64.
-// For a boundary of M = M1 M2 points, X[k1 + M1 k2] = sum_{n2} W^{M1 n2 k2}
-// [W^{n2 k1} sum_{n1} x[M2 n1 + n2] W^{M2 n1 k1}],  W = e^{-2 pi i / M}
-// (two passes of direct sums of length M1 and M2).  omega' = IDFT(i k X) and
-// H omega_0' = IDFT(|k| X) (signed wavenumber k, Nyquist mode zero), the
-// inverse taken as conj(DFT(conj(.)))/M.  A direct circulant convolution with
-// the derivative kernel (entries up to M/2pi of alternating sign) loses too
-// many digits; the DFT keeps FP64 accuracy in every mode.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int dft_find(const DftJobs& J, int t) {
-  int lo = 0;
-  while (lo + 1 < J.n && t >= J.j[lo + 1].start) ++lo;
-  return lo;
-}
-
-__device__ __forceinline__ double signed_k(int i, int M) {
-  if (2 * i == M) return 0.0;           // Nyquist mode set to zero (even M)
-  return (double)(2 * i < M ? i : i - M);
-}
-
-__device__ __forceinline__ double2 dft_input(const DftJob& jb, const double* __restrict__ xr,
-                                             const double2* __restrict__ xc, int i) {
-  if (jb.mode == 0) return make_double2(xr[jb.off_in + i], 0.0);
-  const double2 X = xc[jb.off_in + i];
-  if (jb.mode == 3) return X;                                    // complex input as is
-  if (jb.mode == 6) {                                            // conj(rho(k) X), eq. filter
-    const int ka = (2 * i <= jb.M) ? i : jb.M - i;               // |k|, Nyquist at M/2
-    const double r = (double)ka / (0.5 * (double)jb.M);
-    const double rho = exp(-36.0 * pow(r, 36.0));
-    return make_double2(rho * X.x, -rho * X.y);
-  }
-  const double k = signed_k(i, jb.M);
-  if (jb.mode == 5) return make_double2(-k * k * X.x, k * k * X.y);   // conj(-k^2 X)
-  if (jb.mode == 7) {                                            // conj(X/(ik)), 0 at k = 0
-    if (k == 0.0) return make_double2(0.0, 0.0);
-    return make_double2(X.y / k, X.x / k);
-  }
-  if (jb.mode == 4) {                                            // conj(-i sgn(k) X)
-    const double sg = (k > 0.0) ? 1.0 : (k < 0.0 ? -1.0 : 0.0);
-    return make_double2(sg * X.y, sg * X.x);
-  }
-  if (jb.mode == 1) return make_double2(-k * X.y, -k * X.x);   // conj(i k X)
-  const double ak = fabs(k);
-  return make_double2(ak * X.x, -ak * X.y);                      // conj(|k| X)
-}
-
-// Each output is summed by DFT_SPLIT consecutive lanes (strided terms, a fixed
-// shuffle tree), so a transform of M points keeps DFT_SPLIT M threads busy.
-__device__ __forceinline__ unsigned dft_group_mask() {
-  const unsigned lane = threadIdx.x & 31;
-  return ((1u << DFT_SPLIT) - 1u) << (lane & ~(unsigned)(DFT_SPLIT - 1));
-}
-
-__device__ __forceinline__ void dft_group_sum(double& sr, double& si) {
-  const unsigned mask = dft_group_mask();
-#pragma unroll
-  for (int o = DFT_SPLIT / 2; o > 0; o >>= 1) {
-    sr += __shfl_xor_sync(mask, sr, o);
-    si += __shfl_xor_sync(mask, si, o);
-  }
-}
-
-// pass A: Y[n2 M1 + k1] = W^{n2 k1} sum_{n1} x[M2 n1 + n2] W^{M2 n1 k1}
-__global__ void k_dft_a(DftJobs J, const double* __restrict__ xr, const double2* __restrict__ xc,
-                        const double2* __restrict__ tw, double2* __restrict__ Y,
-                        long long in_stride, long long out_stride) {
-  const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = (int)(gt / DFT_SPLIT), sub = (int)(gt % DFT_SPLIT);
-  if (t >= J.total) return;   // whole groups leave together
-  if (xr) xr += blockIdx.y * in_stride;
-  if (xc) xc += blockIdx.y * in_stride;
-  Y += blockIdx.y * out_stride;
-  const DftJob jb = J.j[dft_find(J, t)];
-  const int q = t - jb.start;
-  const int n2 = q / jb.M1, k1 = q - n2 * jb.M1;
-  const int M = jb.M;
-  const long long step = ((long long)jb.M2 * k1) % M;
-  int idx = (int)((step * sub) % M);
-  const int inc = (int)((step * DFT_SPLIT) % M);
-  double sr = 0.0, si = 0.0;
-  for (int n1 = sub; n1 < jb.M1; n1 += DFT_SPLIT) {
-    const double2 x = dft_input(jb, xr, xc, jb.M2 * n1 + n2);
-    const double2 w = tw[jb.off_tw + idx];
-    sr = fma(x.x, w.x, fma(-x.y, w.y, sr));
-    si = fma(x.x, w.y, fma(x.y, w.x, si));
-    idx += inc;
-    if (idx >= M) idx -= M;
-  }
-  dft_group_sum(sr, si);
-  if (sub == 0) {
-    const double2 w = tw[jb.off_tw + (int)(((long long)n2 * k1) % M)];
-    Y[jb.off_out + q] = make_double2(sr * w.x - si * w.y, sr * w.y + si * w.x);
-  }
-}
-
-// pass B: X[k1 + M1 k2] = sum_{n2} Y[n2 M1 + k1] W^{M1 n2 k2}
-__global__ void k_dft_b(DftJobs J, const double2* __restrict__ Y, const double2* __restrict__ tw,
-                        double2* __restrict__ X, long long stride) {
-  const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int t = (int)(gt / DFT_SPLIT), sub = (int)(gt % DFT_SPLIT);
-  if (t >= J.total) return;
-  Y += blockIdx.y * stride;
-  X += blockIdx.y * stride;
-  const DftJob jb = J.j[dft_find(J, t)];
-  const int q = t - jb.start;
-  const int k2 = q / jb.M1, k1 = q - k2 * jb.M1;
-  const int M = jb.M;
-  const long long step = ((long long)jb.M1 * k2) % M;
-  int idx = (int)((step * sub) % M);
-  const int inc = (int)((step * DFT_SPLIT) % M);
-  double sr = 0.0, si = 0.0;
-  for (int n2 = sub; n2 < jb.M2; n2 += DFT_SPLIT) {
-    const double2 y = Y[jb.off_out + n2 * jb.M1 + k1];
-    const double2 w = tw[jb.off_tw + idx];
-    sr = fma(y.x, w.x, fma(-y.y, w.y, sr));
-    si = fma(y.x, w.y, fma(y.y, w.x, si));
-    idx += inc;
-    if (idx >= M) idx -= M;
-  }
-  dft_group_sum(sr, si);
-  if (sub == 0) X[jb.off_out + q] = make_double2(sr, si);
-}
-
 // spectra -> omega'/M_l (df, all nodes), omega' and H omega_0' (real part / M)
 __global__ void k_dft_extract(Blocks B, const double2* __restrict__ X2, float2* __restrict__ cw,
                               float2* __restrict__ hw0, float* __restrict__ xh,
@@ -396,7 +272,6 @@ bie_status velocity_weights(bie_ctx* c, int nvec, const double* omega, float* xh
   BIE_GET(c, double2, "mdft_Y", (size_t)nvec * (N + M0), dY);
   BIE_GET(c, double2, "mdft_X2", (size_t)nvec * (N + M0), dX2);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "velocity: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
@@ -414,16 +289,10 @@ bie_status velocity_weights(bie_ctx* c, int nvec, const double* omega, float* xh
   J1.total = s1;
   J2.total = s2;
   const long long sY = N + M0;
-  k_dft_a<<<dft_grid(dim3((s1 + 255) / 256, nvec)), 256, 0, c->stream>>>(J1, omega, nullptr, tw, dY, N, sY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
   // every vector's work arrays have stride N + M0; the spectra of the first
   // pair of passes go to X2, which the second pair reads and then overwrites
-  k_dft_b<<<dft_grid(dim3((s1 + 255) / 256, nvec)), 256, 0, c->stream>>>(J1, dY, tw, dX2, sY);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid(dim3((s2 + 255) / 256, nvec)), 256, 0, c->stream>>>(J2, nullptr, dX2, tw, dY, sY, sY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(dim3((s2 + 255) / 256, nvec)), 256, 0, c->stream>>>(J2, dY, tw, dX2, sY);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX2, nvec, N, sY)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX2, dY, dX2, nvec, sY, sY)) return sd;
   const long long next = c->ld + M0;
   k_dft_extract<<<dim3((unsigned)((next + 255) / 256), nvec), 256, 0, c->stream>>>(
       B, dX2, nullptr, hw0, xh, xl, nullptr, c->ld);
@@ -473,7 +342,6 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi)
   BIE_GET(c, double2, "dft_X1", N, dX1);
   BIE_GET(c, double2, "dft_X2", N + M0, dX2);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   const float2* Ttab = (const float2*)ctx_buf(c, "Ttab", sizeof(float2) * M0, &oom);
   const float4* nP = (const float4*)ctx_buf(c, "nP", sizeof(float4) * N, &oom);
   const float4* nQ = (const float4*)ctx_buf(c, "nQ", sizeof(float4) * N, &oom);
@@ -500,15 +368,9 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi)
   s2 += M0;
   J1.total = s1;
   J2.total = s2;
-  k_dft_a<<<dft_grid((s1 + 255) / 256), 256, 0, c->stream>>>(J1, omega, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid((s1 + 255) / 256), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX1)) return sd;
   // inverse of (i k X) per boundary and of (|k| X_0), as conj(DFT(conj(.)))
-  k_dft_a<<<dft_grid((s2 + 255) / 256), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid((s2 + 255) / 256), 256, 0, c->stream>>>(J2, dY, tw, dX2);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   const bool useV = c->assembled;
   float *vxh = nullptr, *vxl = nullptr;
   double* vwp = nullptr;
@@ -759,10 +621,9 @@ extern "C" bie_status bie_normal_velocity_static(int nb, const int* M_host, cons
   s2 += M0;
   J1.total = s1;
   J2.total = s2;
-  k_dft_a<<<dft_grid((s1 + 255) / 256), 256, 0, st>>>(J1, omega_dev, nullptr, tw, dY);
-  k_dft_b<<<dft_grid((s1 + 255) / 256), 256, 0, st>>>(J1, dY, tw, dX1);
-  k_dft_a<<<dft_grid((s2 + 255) / 256), 256, 0, st>>>(J2, nullptr, dX1, tw, dY);
-  k_dft_b<<<dft_grid((s2 + 255) / 256), 256, 0, st>>>(J2, dY, tw, dX2);
+  if (dft_run_plain(st, J1, omega_dev, nullptr, tw, dY, dX1) != cudaSuccess ||
+      dft_run_plain(st, J2, nullptr, dX1, tw, dY, dX2) != cudaSuccess)
+    return BIE_ERR_CUDA;
   k_dft_extract<<<(unsigned)((N + M0 + 255) / 256), 256, 0, st>>>(B, dX2, cw, hw0, nullptr, nullptr,
                                                                   nullptr, ld);
   const int nchunk = (int)((N + VEL_CH - 1) / VEL_CH);
@@ -822,7 +683,6 @@ extern "C" bie_status bie_pressure_rhs(bie_ctx* c, const double* phit, const dou
   BIE_GET(c, double2, "prs_X1", M0, dX1);
   BIE_GET(c, double2, "prs_X2", M0, dX2);
   bool oom = false;
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   const double2* z64 = (const double2*)ctx_buf(c, "zeta", sizeof(double2) * N, &oom);
   const double2* dz64 = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
   const double2* d2z64 = (const double2*)ctx_buf(c, "d2zeta", sizeof(double2) * N, &oom);
@@ -835,15 +695,8 @@ extern "C" bie_status bie_pressure_rhs(bie_ctx* c, const double* phit, const dou
   J1.j[J1.n++] = DftJob{M0, M1, M0 / M1, 0, 0, 0, 0, 0};
   J2.j[J2.n++] = DftJob{M0, M1, M0 / M1, 0, 0, 0, 1, 0};
   J1.total = J2.total = M0;
-  const unsigned gb = (unsigned)((M0 + 255) / 256);
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J1, phit, nullptr, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
-  k_dft_a<<<dft_grid(gb), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-  BIE_LAUNCH_CHECK(c, "k_dft_a");
-  k_dft_b<<<dft_grid(gb), 256, 0, c->stream>>>(J2, dY, tw, dX2);
-  BIE_LAUNCH_CHECK(c, "k_dft_b");
+  if (bie_status sd = dft_run(c, J1, phit, nullptr, dY, dX1)) return sd;
+  if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   k_pressure_rhs<<<obs_grid(N), NODE_THREADS, 0, c->stream>>>(N, M0, make_flow(c), dX2, z64, dz64, d2z64,
                                                          U, tau, g, b);
   BIE_LAUNCH_CHECK(c, "k_pressure_rhs");

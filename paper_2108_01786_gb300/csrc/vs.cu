@@ -225,7 +225,6 @@ extern "C" bie_status bie_vs_normal_velocity(bie_ctx* c, const double* gamma0, d
   const float4* nPQc = (const float4*)ctx_buf(c, "nPQc", sizeof(float4) * N, &oom);
   const double2* z64 = (const double2*)ctx_buf(c, "zeta", sizeof(double2) * N, &oom);
   const double2* dz64 = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
-  const double2* tw = (const double2*)ctx_buf(c, "dft_tw", sizeof(double2) * N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "bie_vs_normal_velocity: node buffers");
   // 1. right-hand side of the solid system
   const int nch = (M0 + VS_CH - 1) / VS_CH;
@@ -270,15 +269,8 @@ extern "C" bie_status bie_vs_normal_velocity(bie_ctx* c, const double* gamma0, d
     J1.j[J1.n++] = DftJob{M0, m1, M0 / m1, 0, 0, 0, 0, 0};
     J2.j[J2.n++] = DftJob{M0, m1, M0 / m1, 0, 0, 0, 4, 0};
     J1.total = J2.total = M0;
-    const unsigned g = (unsigned)((M0 + 255) / 256);
-    k_dft_a<<<dft_grid(g), 256, 0, c->stream>>>(J1, gamma0, nullptr, tw, dY);
-    BIE_LAUNCH_CHECK(c, "k_dft_a");
-    k_dft_b<<<dft_grid(g), 256, 0, c->stream>>>(J1, dY, tw, dX1);
-    BIE_LAUNCH_CHECK(c, "k_dft_b");
-    k_dft_a<<<dft_grid(g), 256, 0, c->stream>>>(J2, nullptr, dX1, tw, dY);
-    BIE_LAUNCH_CHECK(c, "k_dft_a");
-    k_dft_b<<<dft_grid(g), 256, 0, c->stream>>>(J2, dY, tw, dX2);
-    BIE_LAUNCH_CHECK(c, "k_dft_b");
+    if (bie_status sd = dft_run(c, J1, gamma0, nullptr, dY, dX1)) return sd;
+    if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   }
   float2 *cw, *hw0;
   BIE_GET(c, float2, "vel_cw", N, cw);
