@@ -16,7 +16,7 @@
 // X_k = c_k sum_n (x_n c_n) conj(c_{k - n}), a convolution by two transforms of
 // length Q = 2^q >= 2 M - 1 against the tabulated transform of conj(c).
 // Measured: velocity weights at 16383 unknowns (four passes) 88 -> 43 us; a
-// derivative of 3001 (prime) points 249 -> 64 us.
+// derivative of 3001 (prime) points 249 -> 67 us.
 //
 // Modes other than plain input scale the spectrum on the way in; the inverse is
 // conj(DFT(conj(.)))/M, the division left to the caller.  A direct circulant
