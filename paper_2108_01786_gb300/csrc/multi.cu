@@ -376,8 +376,8 @@ struct MArgs {
   double* cs;        // [nrhs][m]
   double* sn;        // [nrhs][m]
   double* g;         // [nrhs][m+1]
-  double* part1;     // [nrhs][m+2][BIE_PSTRIDE]
-  double* part2;     // [nrhs][m+2][BIE_PSTRIDE]
+  double* part1;     // [nrhs][slice][m + 2 + M_RQ]
+  double* part2;     // [nrhs][slice][m + 2 + M_RQ]
   double* partn;     // [nrhs][BIE_NPART]
   MStat* st;         // device
   MStat* mirror;     // host-mapped
@@ -401,7 +401,7 @@ struct MArgs {
   double* Bm;        // [nrhs][m][M_RQ]: C-part of Hessenberg column j
   double* c0;        // [nrhs][M_RQ]: C-part of the cycle's start vector
   double* umean;     // [nrhs][M_RQ][BIE_MAXB]: means of U's columns over the obstacles
-  double* partc;     // [nrhs][M_RQ][BIE_PSTRIDE]: C_i^T r over the slices
+  double* partc;     // [nrhs][slice][M_RQ]: C_i^T r over the slices
 };
 
 __device__ __forceinline__ int mq_of(const MArgs& a, int rr) { return a.st[rr].qc[a.cycle & 1]; }
@@ -414,8 +414,8 @@ __device__ __forceinline__ float* mU(const MArgs& a, int rr, int i) {
 
 // this CTA's slice sums of v over each obstacle, for the next product
 __device__ __forceinline__ void m_obstacle_sums(const MArgs& a, int rr, const float* v, int r0,
-                                                int r1) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+                                                int r1, int nw) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = warp; k < a.nobs; k += nw) {
     const int a0 = max(r0, a.obs_off[k]), a1 = min(r1, a.obs_off[k + 1]);
     double t = 0.0;
@@ -428,6 +428,9 @@ __device__ __forceinline__ void m_obstacle_sums(const MArgs& a, int rr, const fl
 __device__ __forceinline__ float* mV(const MArgs& a, int r, int i) {
   return a.V + ((size_t)r * (a.m + 1) + i) * a.ld;
 }
+
+// doubles between two slices' partial sums in part1, part2
+__device__ __forceinline__ int m_pitch(const MArgs& a) { return a.m + 2 + M_RQ; }
 
 // basis vector i of column rr's cycle: C_i (i < q), V_{i-q}
 __device__ __forceinline__ const float* mQ(const MArgs& a, int rr, int q, int i) {
@@ -496,9 +499,33 @@ __global__ void k_m_resid_finish(MArgs a, const double* __restrict__ ypart, int 
       double t = 0.0;
       for (int m = r0 + lane; m < r1; m += 32) t += (double)ci[m] * rc[m];
       t = warp_sum(t);
-      if (lane == 0) a.partc[((size_t)rr * M_RQ + i) * BIE_PSTRIDE + blockIdx.x] = t;
+      if (lane == 0) a.partc[((size_t)rr * BIE_PSTRIDE + blockIdx.x) * M_RQ + i] = t;
     }
   }
+}
+
+// out[i] = sum of the partials p[c][i], c < np, in a fixed order (i < cnt <= 128): rows in
+// lanes, slices over the warps, about np + 8 FP64 additions per 32 rows where a warp per
+// row and its shuffle tree took 13 instructions for each: FP64 issue (two lanes a cycle
+// per SM, four CTAs) bounded the Gram-Schmidt kernels.  12 columns of 5887 unknowns:
+// k_m_cgs2 11.1 -> 7.4 us a step, k_m_cgs3 13.9 -> 11.5 (its Hessenberg column on a warp of its
+// own as well).  Ends with a barrier; red: 8 x 128 doubles.
+__device__ __forceinline__ void m_reduce(const double* __restrict__ p, int pitch, int cnt, int np,
+                                         double* __restrict__ red, double* __restrict__ out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int i = lane; i < cnt; i += 32) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = warp; c < np; c += nw) s += p[(size_t)c * pitch + i];
+    red[warp * 128 + i] = s;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+    double s = red[i];
+    for (int k = 1; k < nw; ++k) s += red[k * 128 + i];
+    out[i] = s;
+  }
+  __syncthreads();
 }
 
 // ||r||, c_0 = C^T r / ||r||, and v_0 = (r / ||r|| - C c_0) / nu_0 with
@@ -506,7 +533,7 @@ __global__ void k_m_resid_finish(MArgs a, const double* __restrict__ ypart, int 
 __global__ void k_m_start(MArgs a, double rtol, double inner_tol, int first, int max_reached,
                           const int* __restrict__ err) {
   __shared__ double tot, s_nu0;
-  __shared__ double sc[M_RQ];
+  __shared__ double sc[M_RQ], ci[M_RQ], red[8 * 128];
   const int rr = blockIdx.y;
   MStat* S = a.st + rr;
   if (blockIdx.x == 0 && rr == 0 && threadIdx.x == 0) {   // a product's wait ran out: the host stops
@@ -521,13 +548,15 @@ __global__ void k_m_start(MArgs a, double rtol, double inner_tol, int first, int
     s = warp_sum(s);
     if (threadIdx.x == 0) tot = s;
   }
-  if (q > 0) reduce_partials(a.partc + (size_t)rr * M_RQ * BIE_PSTRIDE, q, gridDim.x, sc);
+  if (q > 0) m_reduce(a.partc + (size_t)rr * M_RQ * BIE_PSTRIDE, M_RQ, q, gridDim.x, red, sc);
   __syncthreads();
   const double rn = sqrt(tot);
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int i = 0; i < q; ++i) t += (sc[i] / rn) * (sc[i] / rn);
     s_nu0 = sqrt(fmax(1.0 - t, 0.0));
+  } else if (threadIdx.x >= 32 && (int)threadIdx.x - 32 < q) {
+    ci[threadIdx.x - 32] = sc[threadIdx.x - 32] * (1.0 / rn);
   }
   __syncthreads();
   const double nu0 = s_nu0;
@@ -544,11 +573,18 @@ __global__ void k_m_start(MArgs a, double rtol, double inner_tol, int first, int
     float* v0 = mV(a, rr, 0);
     for (int m = r0 + threadIdx.x; m < r1; m += blockDim.x) {
       double v = a.r[(size_t)rr * a.ld + m] * inv;
-      for (int i = 0; i < q; ++i) v -= (sc[i] * inv) * (double)mC(a, rr, i)[m];
+      for (int i0 = 0; i0 < q; i0 += 8) {   // eight loads in flight
+        float cv[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) cv[u] = i0 + u < q ? mC(a, rr, i0 + u)[m] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (i0 + u < q) v -= ci[i0 + u] * (double)cv[u];
+      }
       v0[m] = (float)(v * inu);
     }
     __syncthreads();
-    m_obstacle_sums(a, rr, v0, r0, r1);
+    m_obstacle_sums(a, rr, v0, r0, r1, blockDim.x >> 5);
   }
   __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -600,13 +636,29 @@ __device__ __forceinline__ double m_lane_dot(const float* va, const float* vb, i
   return s + (double)run;
 }
 
+// Partial dots over this CTA's rows, p[slice][i] = Q_i . w for i < nv (and w . w as
+// i = nv with `norm`), a warp per vector.  (Eight vectors per warp with one exchange
+// tree for their sums takes a quarter of the FP64 additions but leaves most warps
+// idle: 6.8 -> 11.9 us in k_m_finish_dots, 12 columns of 5887 unknowns.)
+__device__ __forceinline__ void m_dots(const MArgs& a, int rr, int q, int nv, bool norm,
+                                       const float* w, int r0, int r1, double* p) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int i = warp; i < nv + (norm ? 1 : 0); i += nw) {
+    double s = m_lane_dot(i < nv ? mQ(a, rr, q, i) : w, w, r0, r1, lane);
+    s = warp_sum(s);
+    if (lane == 0) p[(size_t)blockIdx.x * m_pitch(a) + i] = s;
+  }
+}
+
 // w = D(s v_j + (1/mmin) sum_ks Yp) (+ 3/2 mu_k on obstacle k's rows: A P v_j
-// with A 1_k = -1_k) and part1[i][slice] = V_i . w (i <= j)
+// with A 1_k = -1_k) and part1[slice][i] = Q_i . w (Q = [C, V_0..V_j])
 __global__ void k_m_finish_dots(MArgs a, int j, const float* __restrict__ Yp, int split, int NR,
                                 float inv_mmin) {
   const int rr = blockIdx.y;
   if (a.st[rr].inner_done) return;
   __shared__ float s_xc[BIE_MAXB];
+  int r0, r1;
+  slice_of(a.N, r0, r1);
   {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < a.nobs) {   // means of v_j over the obstacles, in a fixed order
@@ -622,8 +674,6 @@ __global__ void k_m_finish_dots(MArgs a, int j, const float* __restrict__ Yp, in
     }
     __syncthreads();
   }
-  int r0, r1;
-  slice_of(a.N, r0, r1);
   const float* vj = mV(a, rr, j);
   float* w = a.w + (size_t)rr * a.ld;
   for (int m = r0 + threadIdx.x; m < r1; m += blockDim.x) {
@@ -639,14 +689,23 @@ __global__ void k_m_finish_dots(MArgs a, int j, const float* __restrict__ Yp, in
     w[m] = v;
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int q = mq_of(a, rr);
-  double* p1 = a.part1 + (size_t)rr * (a.m + 2 + M_RQ) * BIE_PSTRIDE;
-  for (int i = warp; i <= q + j; i += nw) {
-    double s = m_lane_dot(mQ(a, rr, q, i), w, r0, r1, lane);
-    s = warp_sum(s);
-    if (lane == 0) p1[(size_t)i * BIE_PSTRIDE + blockIdx.x] = s;
+  m_dots(a, rr, q, q + j + 1, false, w, r0, r1, a.part1 + (size_t)rr * m_pitch(a) * BIE_PSTRIDE);
+}
+
+// acc - sum_{i<=nd} h[i] Q_i[m] in the order i = 0 .. nd, eight loads in flight
+__device__ __forceinline__ float m_subtract(const MArgs& a, int rr, int q, int nd, float acc,
+                                            const float* h, int m) {
+  int i = 0;
+  for (; i + 7 <= nd; i += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = mQ(a, rr, q, i + u)[m];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc -= h[i + u] * v[u];
   }
+  for (; i <= nd; ++i) acc -= h[i] * mQ(a, rr, q, i)[m];
+  return acc;
 }
 
 // h1 = sum part1; w' = w - Q h1; part2 = Q^T w' and ||w'||^2 (Q = [C, V_0..V_j])
@@ -655,28 +714,20 @@ __global__ void k_m_cgs2(MArgs a, int j) {
   if (a.st[rr].inner_done) return;
   extern __shared__ double msh[];
   const int q = mq_of(a, rr), nd = q + j;
-  const double* p1 = a.part1 + (size_t)rr * (a.m + 2 + M_RQ) * BIE_PSTRIDE;
-  double* p2 = a.part2 + (size_t)rr * (a.m + 2 + M_RQ) * BIE_PSTRIDE;
+  const double* p1 = a.part1 + (size_t)rr * m_pitch(a) * BIE_PSTRIDE;
+  double* p2 = a.part2 + (size_t)rr * m_pitch(a) * BIE_PSTRIDE;
+  __shared__ double red[8 * 128];
   __shared__ float hf[M_RQ + 66];   // h1 in single precision, converted once per CTA
-  reduce_partials(p1, nd + 1, gridDim.x, msh);
-  __syncthreads();
-  for (int i = threadIdx.x; i <= nd; i += blockDim.x) hf[i] = (float)msh[i];
-  __syncthreads();
   int r0, r1;
   slice_of(a.N, r0, r1);
   float* w = a.w + (size_t)rr * a.ld;
-  for (int m = r0 + threadIdx.x; m < r1; m += blockDim.x) {
-    float acc = w[m];
-    for (int i = 0; i <= nd; ++i) acc -= hf[i] * mQ(a, rr, q, i)[m];
-    w[m] = acc;
-  }
+  m_reduce(p1, m_pitch(a), nd + 1, gridDim.x, red, msh);
+  for (int i = threadIdx.x; i <= nd; i += blockDim.x) hf[i] = (float)msh[i];
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int i = warp; i <= nd + 1; i += nw) {
-    double s = m_lane_dot(i <= nd ? mQ(a, rr, q, i) : w, w, r0, r1, lane);
-    s = warp_sum(s);
-    if (lane == 0) p2[(size_t)i * BIE_PSTRIDE + blockIdx.x] = s;
-  }
+  for (int m = r0 + threadIdx.x; m < r1; m += blockDim.x)
+    w[m] = m_subtract(a, rr, q, nd, w[m], hf, m);
+  __syncthreads();
+  m_dots(a, rr, q, nd + 1, true, w, r0, r1, p2);
 }
 
 // h2 = sum part2, beta, v_{j+1} = (w' - Q h2) / beta; CTA 0: the V-part of
@@ -684,14 +735,22 @@ __global__ void k_m_cgs2(MArgs a, int j) {
 __global__ void k_m_cgs3(MArgs a, int j) {
   const int rr = blockIdx.y;
   MStat* S = a.st + rr;
-  if (S->inner_done) return;
+  // CTA 0 ends the column's cycle below while other CTAs may only be starting: a cycle
+  // that ended at this step (iters = j + 1) still forms its v_{j+1}
+  if (*(volatile int*)&S->inner_done) {
+    __threadfence();
+    if (*(volatile int*)&S->iters <= j) return;
+  }
   extern __shared__ double msh[];
   const int q = mq_of(a, rr), nd = q + j;
-  const double* p1 = a.part1 + (size_t)rr * (a.m + 2 + M_RQ) * BIE_PSTRIDE;
-  const double* p2 = a.part2 + (size_t)rr * (a.m + 2 + M_RQ) * BIE_PSTRIDE;
-  reduce_partials(p2, nd + 2, gridDim.x, msh);
-  if (blockIdx.x == 0) reduce_partials(p1, nd + 1, gridDim.x, msh + (nd + 2));
-  __syncthreads();
+  const double* p1 = a.part1 + (size_t)rr * m_pitch(a) * BIE_PSTRIDE;
+  const double* p2 = a.part2 + (size_t)rr * m_pitch(a) * BIE_PSTRIDE;
+  int r0, r1;
+  slice_of(a.N, r0, r1);
+  const float* w = a.w + (size_t)rr * a.ld;
+  __shared__ double red[8 * 128];
+  m_reduce(p2, m_pitch(a), nd + 2, gridDim.x, red, msh);
+  if (blockIdx.x == 0) m_reduce(p1, m_pitch(a), nd + 1, gridDim.x, red, msh + (nd + 2));
   __shared__ double s_beta;   // sqrt(||w'||^2 - ||h2||^2), one warp's sum for the CTA
   __shared__ float hf[M_RQ + 66], s_inv;   // h2 and 1/beta in single precision
   if (threadIdx.x < 32) {
@@ -707,37 +766,35 @@ __global__ void k_m_cgs3(MArgs a, int j) {
     for (int i = threadIdx.x - 32; i <= nd; i += blockDim.x - 32) hf[i] = (float)msh[i];
   }
   __syncthreads();
+  // the last warp has no rows: in CTA 0 it forms the Hessenberg column meanwhile
+  const int nrow = blockDim.x - 32;
   const double beta = s_beta;
   const bool breakdown = !(beta > 1e-300) || !isfinite(beta);
-  if (!breakdown) {
+  if (!breakdown && (int)threadIdx.x < nrow) {
     const float inv = s_inv;
-    int r0, r1;
-    slice_of(a.N, r0, r1);
-    const float* w = a.w + (size_t)rr * a.ld;
     float* vn = mV(a, rr, j + 1);
-    for (int m = r0 + threadIdx.x; m < r1; m += blockDim.x) {
-      float acc = w[m];
-      for (int i = 0; i <= nd; ++i) acc -= hf[i] * mQ(a, rr, q, i)[m];
+    for (int m = r0 + threadIdx.x; m < r1; m += nrow) {
+      const float acc = m_subtract(a, rr, q, nd, w[m], hf, m);
       vn[m] = acc * inv;
     }
     if (a.nobs > 0) {
-      __syncthreads();   // the slice of v_{j+1} is this CTA's
-      m_obstacle_sums(a, rr, vn, r0, r1);
+      asm volatile("bar.sync 1, %0;" ::"r"(nrow) : "memory");   // the slice of v_{j+1} is this CTA's
+      m_obstacle_sums(a, rr, vn, r0, r1, nrow >> 5);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x < 32) {   // one warp: Hessenberg column and rotations
-    const int m = a.m;
+  if (blockIdx.x == 0 && (int)threadIdx.x >= nrow) {   // one warp: Hessenberg column and rotations
+    const int m = a.m, lane = threadIdx.x & 31;
     double* H = a.H + (size_t)rr * (m + 1) * m;
     double* cs = a.cs + (size_t)rr * m;
     double* sn = a.sn + (size_t)rr * m;
     double* g = a.g + (size_t)rr * (m + 1);
     double* Hj = H + (size_t)j * (m + 1);
-    for (int i = threadIdx.x; i <= j; i += 32) Hj[i] = msh[nd + 2 + q + i] + msh[q + i];
-    for (int l = threadIdx.x; l < q; l += 32)
+    for (int i = lane; i <= j; i += 32) Hj[i] = msh[nd + 2 + q + i] + msh[q + i];
+    for (int l = lane; l < q; l += 32)
       a.Bm[((size_t)rr * m + j) * M_RQ + l] = msh[nd + 2 + l] + msh[l];
     __syncwarp();
     const double uj = givens_apply_warp(Hj, cs, sn, j);
-    if (threadIdx.x != 0) return;
+    if (lane != 0) return;
     Hj[j] = uj;
     Hj[j + 1] = beta;
     const double rr2 = hypot(Hj[j], Hj[j + 1]);
@@ -757,6 +814,7 @@ __global__ void k_m_cgs3(MArgs a, int j) {
     S->resid_est = est;
     const bool nf = !isfinite(est) || !isfinite(rr2);
     if (nf) S->nonfinite = 1;
+    __threadfence();   // iters before inner_done
     if (nf || breakdown || est <= S->inner_tol || j + 1 >= m) S->inner_done = 1;
     m_mirror(a, rr);
   }
@@ -787,15 +845,36 @@ __global__ void k_m_update(MArgs a) {
   __shared__ double Ri[M_RK * M_RK];   // R^-1 (row i, column c)
   __shared__ double Mq[M_RQ * M_RK];   // -B R^-1
   __shared__ float RiF[M_RK * M_RK], MqF[M_RQ * M_RK];   // their single-precision copies
+  // an extending cycle's R (at most M_RK columns) in shared memory, its diagonal's
+  // reciprocals in rd: the substitutions below are chains of dependent loads
+  __shared__ double Rs[M_RK * M_RK], rd[M_RK];
+  if (ext)
+    for (int t = threadIdx.x; t < k * k; t += blockDim.x) {
+      const int l = t / k, i = t - l * k;   // row i, column l
+      const double v = i <= l ? H[(size_t)l * (m + 1) + i] : 0.0;
+      Rs[l * M_RK + i] = v;
+      if (i == l) rd[i] = 1.0 / v;
+    }
+  __syncthreads();
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     for (int i = k - 1; i >= 0; --i) {
       double s = 0.0;
-      for (int l = i + 1 + lane; l < k; l += 32) s += H[(size_t)l * (m + 1) + i] * y[l];
+      for (int l = i + 1 + lane; l < k; l += 32)
+        s += (ext ? Rs[l * M_RK + i] : H[(size_t)l * (m + 1) + i]) * y[l];
       s = warp_sum(s);
-      if (lane == 0) y[i] = (g[i] - s) / H[(size_t)i * (m + 1) + i];
+      if (lane == 0) y[i] = (g[i] - s) / (ext ? Rs[i * M_RK + i] : H[(size_t)i * (m + 1) + i]);
       __syncwarp();
     }
+  } else if (ext && threadIdx.x >= 32 && (int)threadIdx.x < 32 + k) {   // column c of R^-1
+    const int c = threadIdx.x - 32;
+    for (int i = 0; i < k; ++i) Ri[i * M_RK + c] = 0.0;
+    for (int i = c; i >= 0; --i) {
+      double t = i == c ? 1.0 : 0.0;
+      for (int l = i + 1; l <= c; ++l) t -= Rs[l * M_RK + i] * Ri[l * M_RK + c];
+      Ri[i * M_RK + c] = t * rd[i];
+    }
+    for (int i = 0; i < k; ++i) RiF[i * M_RK + c] = (float)Ri[i * M_RK + c];
   }
   __syncthreads();
   if ((int)threadIdx.x < q) {
@@ -803,16 +882,6 @@ __global__ void k_m_update(MArgs a) {
     double t = a.c0[(size_t)rr * M_RQ + l];
     for (int i = 0; i < k; ++i) t -= Bm[(size_t)i * M_RQ + l] * y[i];
     tq[l] = t;
-  }
-  if (ext && (int)threadIdx.x < k) {   // column c of R^-1
-    const int c = threadIdx.x;
-    for (int i = 0; i < k; ++i) Ri[i * M_RK + c] = 0.0;
-    for (int i = c; i >= 0; --i) {
-      double t = i == c ? 1.0 : 0.0;
-      for (int l = i + 1; l <= c; ++l) t -= H[(size_t)l * (m + 1) + i] * Ri[l * M_RK + c];
-      Ri[i * M_RK + c] = t / H[(size_t)i * (m + 1) + i];
-    }
-    for (int i = 0; i < k; ++i) RiF[i * M_RK + c] = (float)Ri[i * M_RK + c];
   }
   __syncthreads();
   if (ext)
