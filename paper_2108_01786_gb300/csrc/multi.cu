@@ -401,6 +401,9 @@ struct MArgs {
   double* Bm;        // [nrhs][m][M_RQ]: C-part of Hessenberg column j
   double* c0;        // [nrhs][M_RQ]: C-part of the cycle's start vector
   double* umean;     // [nrhs][M_RQ][BIE_MAXB]: means of U's columns over the obstacles
+  void* XT;          // [columns padded][ld]: v_j / M_l * mmin in the storage type, the next product's x
+  int bf;
+  double mmin;
   double* partc;     // [nrhs][slice][M_RQ]: C_i^T r over the slices
 };
 
@@ -435,6 +438,15 @@ __device__ __forceinline__ int m_pitch(const MArgs& a) { return a.m + 2 + M_RQ; 
 // basis vector i of column rr's cycle: C_i (i < q), V_{i-q}
 __device__ __forceinline__ const float* mQ(const MArgs& a, int rr, int q, int i) {
   return i < q ? mC(a, rr, i) : mV(a, rr, i - q);
+}
+
+// row m of the next product's column, written with v_j itself (a kernel of its own per step
+// was 2.2 us and a launch: 12 columns of 5887 unknowns, 21 steps, 2288 us with it, now 2204)
+__device__ __forceinline__ void m_store_x(const MArgs& a, int rr, int m, float v) {
+  const size_t i = (size_t)rr * a.ld + m;
+  const float t = (float)((double)v * a.wgt64[m] * a.mmin);
+  if (a.bf) ((__nv_bfloat16*)a.XT)[i] = __float2bfloat16_rn(t);
+  else ((__half*)a.XT)[i] = __float2half_rn(t);
 }
 
 __device__ __forceinline__ void m_mirror(const MArgs& a, int r) {
@@ -582,6 +594,7 @@ __global__ void k_m_start(MArgs a, double rtol, double inner_tol, int first, int
           if (i0 + u < q) v -= ci[i0 + u] * (double)cv[u];
       }
       v0[m] = (float)(v * inu);
+      m_store_x(a, rr, m, v0[m]);
     }
     __syncthreads();
     m_obstacle_sums(a, rr, v0, r0, r1, blockDim.x >> 5);
@@ -603,20 +616,6 @@ __global__ void k_m_start(MArgs a, double rtol, double inner_tol, int first, int
     for (int i = 0; i < q; ++i) a.c0[(size_t)rr * M_RQ + i] = sc[i] / rn;
     m_mirror(a, rr);
   }
-}
-
-// XT[rr][l] = v_j^rr[l] / M_l * mmin in the storage type (zero for finished or padding columns)
-template <bool BF16>
-__global__ void k_m_prep(MArgs a, int j, int NR, double mmin, void* __restrict__ XT) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)NR * a.ld) return;
-  const int rr = (int)(i / a.ld);
-  const int l = (int)(i - (long long)rr * a.ld);
-  float v = 0.f;
-  if (rr < a.nrhs && l < a.N && !a.st[rr].inner_done)
-    v = (float)((double)mV(a, rr, j)[l] * a.wgt64[l] * mmin);
-  if (BF16) ((__nv_bfloat16*)XT)[i] = __float2bfloat16_rn(v);
-  else ((__half*)XT)[i] = __float2half_rn(v);
 }
 
 // this lane's share of a . b over the slice: FP32 runs of eight, the runs in FP64
@@ -775,7 +774,9 @@ __global__ void k_m_cgs3(MArgs a, int j) {
     float* vn = mV(a, rr, j + 1);
     for (int m = r0 + threadIdx.x; m < r1; m += nrow) {
       const float acc = m_subtract(a, rr, q, nd, w[m], hf, m);
-      vn[m] = acc * inv;
+      const float v = acc * inv;
+      vn[m] = v;
+      m_store_x(a, rr, m, v);
     }
     if (a.nobs > 0) {
       asm volatile("bar.sync 1, %0;" ::"r"(nrow) : "memory");   // the slice of v_{j+1} is this CTA's
@@ -1263,6 +1264,11 @@ bie_status solve_multi_run(bie_ctx* c, int nrhs, int rhs_kind, const double* rhs
   BIE_CUDA_TRY(c, cudaMemsetAsync(X, 0, sizeof(double) * (size_t)nrhs * N, c->stream));
   BIE_CUDA_TRY(c, cudaMemsetAsync(st, 0, sizeof(MStat) * nrhs, c->stream));
   BIE_CUDA_TRY(c, cudaMemsetAsync(err, 0, sizeof(int), c->stream));
+  // the padding rows and columns of the products' x stay zero
+  BIE_CUDA_TRY(c, cudaMemsetAsync(XT, 0, sizeof(unsigned short) * (size_t)NR * ld, c->stream));
+  a.XT = XT;
+  a.bf = bf ? 1 : 0;
+  a.mmin = (double)mmin;
   double inner_tol = o->inner_tol;
   // Up to 16 columns the recycled space pays (26 -> 21 steps, 4 cycles instead of
   // 5); with more, the per-column Gram-Schmidt work over the extra basis vectors
@@ -1287,10 +1293,6 @@ bie_status solve_multi_run(bie_ctx* c, int nrhs, int rhs_kind, const double* rhs
   BIE_CUDA_TRY(c, cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
 
   auto step = [&](int j) -> bie_status {
-    const unsigned gp = (unsigned)(((long long)NR * ld + 255) / 256);
-    if (bf) k_m_prep<true><<<gp, 256, 0, c->stream>>>(a, j, NR, (double)mmin, XT);
-    else k_m_prep<false><<<gp, 256, 0, c->stream>>>(a, j, NR, (double)mmin, XT);
-    BIE_LAUNCH_CHECK(c, "k_m_prep");
     bie_status s;
     if (NR == 16) s = bf ? mm_launch<16, 6, true>(c, tA, tX, Yp, split, err) : mm_launch<16, 6, false>(c, tA, tX, Yp, split, err);
     else if (NR == 32) s = bf ? mm_launch<32, 6, true>(c, tA, tX, Yp, split, err) : mm_launch<32, 6, false>(c, tA, tX, Yp, split, err);
