@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -25,3 +26,10 @@ def pytest_collection_modifyitems(config, items):
     for it in items:
         if "gpu" in it.keywords:
             it.add_marker(skip)
+
+
+def pytest_runtest_setup(item):
+    # tensors that earlier tests left in reference cycles go now, not in the middle of
+    # a test that compares allocated bytes
+    if item.get_closest_marker("gpu"):
+        gc.collect()
