@@ -269,11 +269,13 @@ struct bie_ctx {
   void* exch_buf = nullptr;      // caller's staging buffer
   size_t exch_bytes = 0;
 
-  // exchange buffers of the one-kernel solver (resident.cu) that were last zeroed
+  // exchange buffers of the one-kernel solver (resident.cu) that were last zeroed,
+  // and the sizes (leading dimension, unknowns, bytes per element) they were zeroed for
   const void* rs_bar = nullptr;
   const void* rs_x = nullptr;
   long long rs_ld = 0;
   int rs_n = 0;
+  int rs_vt = 0;
 
   // named device buffers
   std::vector<std::pair<std::string, DevBuf>> bufs;

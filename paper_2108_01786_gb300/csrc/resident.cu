@@ -1416,10 +1416,13 @@ bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const
     BIE_CUDA_TRY(c, cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), c->stream));
     c->rs_bar = bar;
   }
-  if (c->rs_ld != c->ld || c->rs_n != c->N || c->rs_x != xb) {   // the padding past N stays zero
+  // The padding past N stays zero: N, ld and the element width say where it lies (the
+  // FP64 scheme's doubles cover what are padding floats of a refined solve)
+  if (c->rs_ld != c->ld || c->rs_n != c->N || c->rs_vt != (int)vt || c->rs_x != xb) {
     BIE_CUDA_TRY(c, cudaMemsetAsync(xb, 0, 3 * ldb, c->stream));
     c->rs_ld = c->ld;
     c->rs_n = c->N;
+    c->rs_vt = (int)vt;
     c->rs_x = xb;
   }
   a.zbuf = xb;

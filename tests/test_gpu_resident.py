@@ -115,3 +115,57 @@ def test_one_kernel_solve_guesses_zero_and_nonfinite(P, prec):
             assert float((x / s - prob.omega).norm() / prob.omega.norm()) <= 1e-12
     finally:
         prob.close()
+
+
+def test_precision_change_on_one_context(P):
+    """The schemes share the solver's exchange buffers, whose padding past N must read as
+    zero.  The FP64 solve here leaves doubles whose low words are NaN as floats where
+    the refined schemes have their padding: x is the solution already, so x / M_l is
+    published once (1 / M_l a power of two keeps the low words) and nothing after it."""
+    import torch
+    g, f, ph = _geometry(64, 32, [9])
+    assert g.N == 105                        # floats 105 .. 127 overlay doubles 52 .. 63, surface nodes
+    x = np.random.default_rng(5).standard_normal(g.N)
+    low = x.view(np.uint64) & np.uint64(0xffffffff00000000)
+    x = (low | np.uint64(0x7fc00001)).view(np.float64)
+    xd = torch.as_tensor(x, device="cuda")
+    prob = P.Problem(g, f, ph)
+    try:
+        for prec in ("fp32_ir", "fp16_ir", "bf16_ir"):
+            prob.assemble("fp64")
+            b = torch.empty_like(xd)
+            P.bie_matvec(prob.ctx, 1, xd, b)
+            om = xd.clone()
+            info = P.bie_solve_b(prob.ctx, b, om, P.bie_default_opts(x0=1, rtol=1e-10))
+            assert info.cycles == 0 and torch.equal(om, xd)
+            prob.assemble(prec)
+            info = P.bie_solve_b(prob.ctx, b, om)
+            assert info.converged
+            other = P.Problem(g, f, ph)      # a context that never solved in FP64
+            try:
+                other.assemble(prec)
+                want = torch.empty_like(om)
+                P.bie_solve_b(other.ctx, b, want)
+                assert torch.equal(om, want), prec
+            finally:
+                other.close()
+    finally:
+        prob.close()
+
+
+@pytest.mark.parametrize("n", [1001, 4099])
+def test_fp64_then_refined_on_one_context(P, n):
+    g, f, ph = W.random_geometry(np.random.default_rng(n), n)
+    prob = P.Problem(g, f, ph)
+    try:
+        for seed in range(6):
+            prob.phit.copy_(prob.phit.new_tensor(W.filtered_noise(np.random.default_rng(seed), g.M[0], 0.05, 8)))
+            prob.assemble("fp64")
+            assert prob.solve().converged
+            ref = prob.omega.clone()
+            for prec in ("fp32_ir", "fp16_ir", "bf16_ir"):
+                prob.assemble(prec)
+                assert prob.solve().converged
+                assert float((prob.omega - ref).norm() / ref.norm()) <= 1e-12
+    finally:
+        prob.close()
