@@ -253,11 +253,8 @@ __global__ void __launch_bounds__(PSUM_THREADS, 3)
                        : d2_dot2<false>(Wr, dr, Wi, di, f2(0.f), f2(0.f));
       a2 = d2_macc(a2, v, inv);
       if (same) {   // T_0 = 0: the target itself drops out
-        int ia = idx + p;
-        ia -= ia >= Mk ? Mk : 0;
-        int ib = ia + 16;
-        ib -= ib >= Mk ? Mk : 0;
-        const float2 ta = nd.Tall[om + ia], tb = nd.Tall[om + ib];
+        const float2 ta = nd.Tall[om + psum_index_up(idx, p, n, Mk)];
+        const float2 tb = nd.Tall[om + psum_index_up(idx, p + 16, n, Mk)];
         at = d2_macc(at, df2{f2(ta.x, tb.x), f2(ta.y, tb.y)}, d2_of(S[sl].W[2][p]));
       }
     }

@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "pair_kernel.cuh"
 #include "df2.cuh"
+#include "psum_index.h"
 
 #define PSUM_WARPS 8
 #define PSUM_THREADS (32 * PSUM_WARPS)

@@ -83,11 +83,8 @@ __global__ void __launch_bounds__(PSUM_THREADS, 2)
       ar = d2_macc(ar, di, q);
       ai = d2_macc(ai, dr, q);
       if (same) {   // T_0 = 0: the target itself drops out
-        int ia = idx - p;
-        ia += ia < 0 ? Mk : 0;
-        int ib = ia - 16;
-        ib += ib < 0 ? Mk : 0;
-        const float2 ta = nd.Tall[om + ia], tb = nd.Tall[om + ib];
+        const float2 ta = nd.Tall[om + psum_index_down(idx, p, n, Mk)];
+        const float2 tb = nd.Tall[om + psum_index_down(idx, p + 16, n, Mk)];
         at = d2_macc(at, df2{f2(ta.x, tb.x), f2(ta.y, tb.y)}, c);
       }
     }

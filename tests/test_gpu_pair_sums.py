@@ -88,3 +88,27 @@ def test_far_targets_do_not_depend_on_their_neighbours(P):
         assert np.abs(full[:200].cpu().numpy() - ref).max() <= 1e-4 * np.abs(ref).max()
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("M0,M1,Mo", [(8, 16, []), (9, 8, [15]), (15, 40, [9, 8]), (64, 15, [16, 8]), (16, 17, [8])])
+def test_boundary_sums_of_short_boundaries(P, M0, M1, Mo):
+    """Boundaries of 8 to 17 nodes, first, last and between: shorter than half a tile."""
+    import torch
+    g, f = _geometry(M0, M1, Mo)
+    om = W.smooth_density(g, seed=2, kmax=2)
+    ph = W.filtered_noise(np.random.default_rng(1), M0, 0.05, 2)
+    prob = P.Problem(g, f, ph)
+    try:
+        omd = torch.as_tensor(om, device="cuda")
+        v = torch.empty(g.N, dtype=torch.complex128, device="cuda")
+        P.bie_boundary_velocity(prob.ctx, omd, v)
+        ref = np.concatenate(O.boundary_dphi(g, f, om))
+        assert np.abs(v.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
+        E = P.bie_energy(prob.ctx, prob.phit, omd, tau=0.1, g=1.0)
+        assert abs(E - O.energy(g, f, ph, om)) <= 1e-10 * max(1.0, abs(E))
+        prob.assemble("fp32_ir")
+        P.bie_boundary_potential(prob.ctx, omd, v)
+        ref = np.concatenate(O.phi_tilde_boundary(g, om))
+        assert np.abs(v.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
+    finally:
+        prob.close()
