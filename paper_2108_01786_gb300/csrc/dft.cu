@@ -9,7 +9,10 @@
 // output count: a pass of length L = La Lb takes La + Lb terms in two steps through
 // shared memory instead of L (8192 points: 16 + 24 instead of 64 + 128), and many
 // small CTAs spread the columns over the chip.  A prime L (or one with a prime
-// factor above 64) is summed directly, its outputs shared by several CTAs.
+// factor above 64) is summed directly, its outputs shared by several CTAs and its
+// input staged DFT_CHUNK elements at a time: with all of it staged, 131 KB at 8179
+// (a length the context-free velocity takes), one CTA of four warps had an SM to
+// itself and waited for its own sums (8179 + 13 nodes: 5365 us, in pieces 2650).
 // Lengths with a large prime factor P, where that still means P terms per output
 // (M P > 2^20), take Bluestein's form (L. Bluestein, "A linear filtering approach to
 // the computation of discrete Fourier transform", 1970): with c_n = e^{-i pi n^2 / M},
@@ -30,6 +33,7 @@
 
 #define DFT_THREADS 128
 #define DFT_TW_SMEM 1024   // transforms up to this length keep their twiddles in shared memory
+#define DFT_CHUNK 512      // input elements of a longer direct pass staged at a time
 
 namespace {
 
@@ -129,32 +133,37 @@ __global__ void __launch_bounds__(DFT_THREADS) k_dft(const __grid_constant__ Dft
   double2* sm = st + (L <= DFT_TW_SMEM ? L : 0);   // first step's result (two-step form)
   if (L <= DFT_TW_SMEM)
     for (int j = threadIdx.x; j < L; j += DFT_THREADS) st[j] = tw[(size_t)j * cols];
-  for (int e = threadIdx.x; e < nc * L; e += DFT_THREADS) {
-    const int n = e / nc, c = e - n * nc;
-    const int i = n * cols + col0 + c;
-    double2 x;
-    switch (p.kind) {
-      case PA_IN:
-        x = dft_input(p.mode, p.T, p.in, a.xr + v * a.in_stride, a.xr2, a.xc + v * a.in_stride, i);
-        break;
-      case PA_BL:
-        x = make_double2(0.0, 0.0);
-        if (i < p.Mt)
-          x = zmul(dft_input(p.mode, p.Mt, p.in, a.xr + v * a.in_stride, a.xr2, a.xc + v * a.in_stride, i),
-                   a.chirp[p.chirp + i]);
-        break;
-      case PA_MID:
-        x = zmul(a.blf[v * a.bl_stride + p.work + i], a.bhat[p.bhat + i]);
-        x.y = -x.y;
-        break;
-      case PB_OUT:
-        x = a.Y[v * a.stride + p.out + i];
-        break;
-      default:
-        x = a.bly[v * a.bl_stride + p.work + i];
+  // elements n0 .. n0 + len - 1 of every column into sx (all of them, but for a long direct pass)
+  const int chunk_len = p.La == 1 && L > DFT_TW_SMEM ? DFT_CHUNK : L;
+  auto stage = [&](int n0, int len) {
+    for (int e = threadIdx.x; e < nc * len; e += DFT_THREADS) {
+      const int n = e / nc, c = e - n * nc;
+      const int i = (n0 + n) * cols + col0 + c;
+      double2 x;
+      switch (p.kind) {
+        case PA_IN:
+          x = dft_input(p.mode, p.T, p.in, a.xr + v * a.in_stride, a.xr2, a.xc + v * a.in_stride, i);
+          break;
+        case PA_BL:
+          x = make_double2(0.0, 0.0);
+          if (i < p.Mt)
+            x = zmul(dft_input(p.mode, p.Mt, p.in, a.xr + v * a.in_stride, a.xr2, a.xc + v * a.in_stride, i),
+                     a.chirp[p.chirp + i]);
+          break;
+        case PA_MID:
+          x = zmul(a.blf[v * a.bl_stride + p.work + i], a.bhat[p.bhat + i]);
+          x.y = -x.y;
+          break;
+        case PB_OUT:
+          x = a.Y[v * a.stride + p.out + i];
+          break;
+        default:
+          x = a.bly[v * a.bl_stride + p.work + i];
+      }
+      sx[n * C + c] = x;
     }
-    sx[n * C + c] = x;
-  }
+  };
+  stage(0, min(L, chunk_len));
   __syncthreads();
   auto W = [&](int j) -> double2 { return L <= DFT_TW_SMEM ? st[j] : tw[(size_t)j * cols]; };
   auto store = [&](int c, int k, double2 x) {
@@ -217,24 +226,30 @@ __global__ void __launch_bounds__(DFT_THREADS) k_dft(const __grid_constant__ Dft
     }
     return;
   }
-  // direct: outputs k0 .. k0 + nk - 1 of every column of the CTA
+  // direct: outputs k0 .. k0 + nk - 1 of the CTA's column, at most one per lane group
   const int k0 = chunk * p.KC, nk = min(p.KC, L - k0), nout = nc * nk;
-  for (int b0 = 0; b0 < nout; b0 += per) {
-    const int e = min(b0 + e0, nout - 1);
-    const int c = p.kind <= PA_MID ? e / nk : e % nc, k = k0 + (p.kind <= PA_MID ? e % nk : e / nc);
-    ZAcc s;
-    s.zero();
-    int j = (int)(((long long)k * sub) % L);
-    const int step = (int)(((long long)k * sp) % L);
+  const int e = min(e0, nout - 1);
+  const int c = p.kind <= PA_MID ? e / nk : e % nc, k = k0 + (p.kind <= PA_MID ? e % nk : e / nc);
+  ZAcc s;
+  s.zero();
+  int j = (int)(((long long)k * sub) % L);
+  const int step = (int)(((long long)k * sp) % L);
+  for (int n0 = 0; n0 < L; n0 += chunk_len) {
+    const int len = min(chunk_len, L - n0);
+    if (n0 > 0) {   // the previous piece has been read
+      __syncthreads();
+      stage(n0, len);
+      __syncthreads();
+    }
 #pragma unroll 4
-    for (int n = sub; n < L; n += sp) {
+    for (int n = sub; n < len; n += sp) {   // a piece's length is a multiple of sp but for the last
       s.add(sx[n * C + c], W(j));
       j += step;
       if (j >= L) j -= L;
     }
-    const double2 x = lanes(s.value());
-    if (sub == 0 && b0 + e0 < nout) store(c, k, x);
   }
+  const double2 x = lanes(s.value());
+  if (sub == 0 && e0 < nout) store(c, k, x);
 }
 
 // c_n = e^{-i pi n^2 / M}, the padded sequence conj(c) (in F) and the twiddles of length Q
@@ -299,7 +314,8 @@ int plan_pass(DftP& p, int T, int L, long long terms, long long cols, size_t* sm
     p.sp = DFT_THREADS / p.KC;
   }
   p.nch = (L + p.KC - 1) / p.KC;
-  const size_t need = (size_t)p.C * L * (p.La > 1 ? 2 : 1) + (L <= DFT_TW_SMEM ? L : 0);
+  const int staged = p.La == 1 && L > DFT_TW_SMEM ? DFT_CHUNK : L;
+  const size_t need = (size_t)p.C * staged * (p.La > 1 ? 2 : 1) + (L <= DFT_TW_SMEM ? L : 0);
   *smem = std::max(*smem, need * sizeof(double2));
   return (p.cols + p.C - 1) / p.C * p.nch;
 }

@@ -68,3 +68,18 @@ def test_several_vectors_of_prime_lengths(P):
             assert np.linalg.norm(V.cpu().numpy() - Uref) <= 1e-11 * np.linalg.norm(Uref)
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("M0,M1", [(1021, 16), (1031, 2053), (2062, 9), (4093, 64)])
+def test_context_free_velocity_of_prime_lengths(P, M0, M1):
+    """The context-free call sums prime lengths directly, longer ones in pieces of 512 with a
+    remainder (1031, 2053, 4093) or not at all (1021)."""
+    import torch
+    g = W.simple_channel(M0, M1)
+    om = W.smooth_density(g, seed=2, kmax=4)
+    c = lambda v: torch.as_tensor(np.asarray(v, dtype=complex), device="cuda")
+    U = torch.empty(M0, dtype=torch.float64, device="cuda")
+    P.bie_normal_velocity_static(list(g.M), c(g.zeta), c(g.dzeta), c(g.d2zeta), None, 0.6, None,
+                                 torch.as_tensor(om, device="cuda"), U)
+    ref = O.normal_velocity(g, W.Flow(V1=0.6, a=np.zeros(0)), om)
+    assert np.linalg.norm(U.cpu().numpy() - ref) <= 1e-11 * np.linalg.norm(ref)
