@@ -1288,12 +1288,16 @@ bie_status bie_batch_set_problem(bie_batch* b, int p, int nb, const int* M_host,
   b->set[p] = 0;
   // the inputs may have been written on the caller's stream
   if (b->user_stream) BT_TRY(b, cudaStreamSynchronize(b->user_stream));
-  const int oldN = c->N;
+  // The captured graph holds addresses of buffers sized by the boundaries' node counts (the
+  // transforms' tables among them), which other counts may reallocate, with the same
+  // total or in a call that then fails: it goes before they do
+  bool same = c->have_geom && nb == c->nb && M_host;
+  for (int k = 0; same && k < nb; ++k) same = M_host[k] == c->M[k];
+  if (!same) bt_drop_graph(b);
   bie_status s = bie_set_geometry(c, nb, M_host, zeta_dev, dzeta_dev, d2zeta_dev, zc_host);
   if (s == BIE_OK) s = bie_set_flow(c, V1, a_host);
   if (s != BIE_OK) return bt_fail(b, s, "problem " + std::to_string(p) + ": " + c->err);
   if (c->N > BT_MAXLD) return bt_fail(b, BIE_ERR_ARG, "bie_batch_set_problem: N > 16384");
-  if (c->N != oldN) bt_drop_graph(b);
   b->set[p] = 1;
   return BIE_OK;
 }

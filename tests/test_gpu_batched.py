@@ -280,3 +280,28 @@ def test_batch_reported_residual_is_the_true_one(P, prec):
         assert lo * sum(ent) <= rb <= 8 * sum(ent), (rb, sum(ent))
     finally:
         bt.close()
+
+
+def test_other_node_counts_of_the_same_total_drop_the_graph(P):
+    """X, run; Y (as many unknowns, longer transform tables), not run; X again, run: the graph
+    captured for X must not be replayed, its tables were reallocated for Y."""
+    import torch
+
+    def channel(M0, M1):
+        g = W.simple_channel(M0=M0, M1=M1, h=1.0)
+        return g, W.Flow(V1=0.9, a=np.array([])), W.filtered_noise(np.random.default_rng(3), M0, 0.05, 16)
+    X, Y = channel(1031, 1100), channel(2053, 78)     # Bluestein lengths 4096 and 8192
+    bt = Batch(P, [X])
+    try:
+        bt.run("fp32_ir")
+        om, U = bt.omega.clone(), bt.U.clone()
+        zt = lambda a: torch.as_tensor(a, dtype=torch.complex128, device="cuda").contiguous()
+        for g, f, _ in (Y, X):            # the run's own buffers stay, as does its key
+            P.bie_batch_set_problem(bt.b, 0, g.M, zt(g.zeta), zt(g.dzeta), zt(g.d2zeta), g.zc, f.V1, f.a)
+        bt.run("fp32_ir")
+        assert float((bt.omega - om).norm() / om.norm()) <= 1e-12
+        assert float((bt.U - U).norm() / U.norm()) <= 1e-12
+        Uref = O.normal_velocity(X[0], X[1], om.cpu().numpy())
+        assert _rel(bt.U.cpu().numpy(), Uref) <= 1e-11
+    finally:
+        bt.close()
