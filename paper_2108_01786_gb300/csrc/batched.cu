@@ -161,10 +161,14 @@ __device__ __forceinline__ bool bt_barrier(unsigned* bar, int* err, unsigned spi
 }
 
 // Thread 0 takes the next unit of the phase and tests its problem's flag
-// (which: 0 none, 1 active, 2 inner); every thread gets the same answer:
-// 0 no unit left, 1 skip, 2 work on *s_unit.
+// (which: 0 none, 1 active, 2 inner, 3 inner when step j began); every thread gets
+// the same answer: 0 no unit left, 1 skip, 2 work on *s_unit.
+// 3: the leader unit clears inner in the phase that also forms v_{j+1}; a unit of the
+// problem taken after that still has rows of it to form (iters = j + 1: the cycle ended
+// at this step; iters is written before inner is cleared).
 __device__ __forceinline__ int bt_take(unsigned* ctr, const BtUnit* units, int count,
-                                       const BtStat* st, int which, BtUnit* s_unit, int* s_state) {
+                                       const BtStat* st, int which, BtUnit* s_unit, int* s_state,
+                                       int j = 0) {
   __syncthreads();
   if (threadIdx.x == 0) {
     const int u = (int)atomicAdd(ctr, 1u);
@@ -172,7 +176,11 @@ __device__ __forceinline__ int bt_take(unsigned* ctr, const BtUnit* units, int c
     if (u < count) {
       const BtUnit U = units[u];
       *s_unit = U;
-      const int f = which == 0 ? 1 : (which == 1 ? __ldcg(&st[U.p].active) : __ldcg(&st[U.p].inner));
+      int f = which == 0 ? 1 : (which == 1 ? __ldcg(&st[U.p].active) : __ldcg(&st[U.p].inner));
+      if (which == 3 && !f) {
+        __threadfence();
+        f = __ldcg(&st[U.p].active) && __ldcg(&st[U.p].iters) == j + 1;
+      }
       state = f ? 2 : 1;
     }
     *s_state = state;
@@ -604,6 +612,7 @@ __device__ void bt_cgs3(const BtArgs& a, const BtProb& P, const BtUnit& U, int p
       S->active = 0;
     }
     const bool end = nf || breakdown || est <= S->inner_tol || j + 1 >= mend;
+    __threadfence();   // iters and active before inner
     if (end) S->inner = 0;
     *s_flag = (end && !nf) ? 1 : 0;
   }
@@ -860,9 +869,9 @@ __global__ void __launch_bounds__(BT_THREADS, 1) k_batch_gmres(BtArgs a, int max
       if (!end_phase()) return;
       begin_phase();
       for (;;) {   // CGS3
-        // the leader may end the cycle while other units of the problem are
-        // in this phase; they then skip v_{j+1}, which the update does not use
-        const int k = bt_take(ctr + (t % 3), a.vunits, a.nvu, a.st, 2, &s_unit, &s_state);
+        // the update takes v_{j+1} of the last step too when the cycle's space joins the
+        // recycled one, so every unit forms it
+        const int k = bt_take(ctr + (t % 3), a.vunits, a.nvu, a.st, 3, &s_unit, &s_state, j);
         if (k == 0) break;
         if (k == 1) continue;
         const BtUnit U = s_unit;

@@ -305,3 +305,21 @@ def test_other_node_counts_of_the_same_total_drop_the_graph(P):
         assert _rel(bt.U.cpu().numpy(), Uref) <= 1e-11
     finally:
         bt.close()
+
+
+def test_more_vector_units_than_sms_give_the_same_bits(P):
+    """More vector units than CTAs: units of one problem are taken at different times of a
+    phase, and a cycle that ends in it ends for all of them at the same step."""
+    rng = np.random.default_rng(5)
+    probs = [W.random_geometry(rng, int(n)) for n in rng.integers(2000, 9000, 40)]
+    assert sum((g.N + 1023) // 1024 for g, _, _ in probs) > 152
+    bt = Batch(P, probs)
+    try:
+        for kw in ({}, {"restart": 4, "max_cycles": 60}):
+            bt.run("fp16_ir", **kw)
+            om, U = bt.omega.clone(), bt.U.clone()
+            for _ in range(9):
+                bt.run("fp16_ir", **kw)
+                assert bool((bt.omega == om).all()) and bool((bt.U == U).all()), kw
+    finally:
+        bt.close()
