@@ -53,7 +53,8 @@
 int gemv_num_ctas();
 
 struct RsOut {            // host-mapped result of a solve
-  int iters, cycles, converged, nonfinite, stagnated, pad;
+  int iters, cycles, converged, nonfinite, stagnated;
+  int timeout;            // set before the launch, cleared by the last CTA out if no wait ran out
   double rnorm, bnorm;
 };
 static_assert(sizeof(RsOut) <= sizeof(HostSlot) * BIE_NSLOTS, "result fits the slot ring");
@@ -570,11 +571,15 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
   }
   auto flip = [&](int t) -> bool { return swt[2 * R + t] < (VT)0; };
   auto qv = [&](int q, int i) -> const VT* { return i < q ? C + (size_t)i * R : V + (size_t)(i - q) * R; };
-  auto leave = [&]() {   // the last CTA out zeroes the barrier for the next solve
+  // The last CTA out zeroes the barrier for the next solve and reports: a CTA may have given
+  // up at a barrier that the others passed, its rows of x then not being the result's.
+  auto leave = [&]() {
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
       if (atomicAdd(a.bar + 1, 1u) == (unsigned)G - 1) {
+        __threadfence();
+        a.out->timeout = *(volatile int*)a.err;
         a.bar[0] = 0;
         a.bar[1] = 0;
         __threadfence();
@@ -1216,16 +1221,14 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
   }
   for (int t = threadIdx.x; t < nr; t += blockDim.x) a.x[c0r + t] = sx[t];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    RsOut o;
-    o.iters = total;
-    o.cycles = cycles;
-    o.converged = s_state == 1;
-    o.nonfinite = s_state == 2 || s_nonf;
-    o.stagnated = s_state == 3;
-    o.pad = 0;
-    o.rnorm = s_rn;
-    o.bnorm = bnorm;
-    *a.out = o;
+    RsOut* o = a.out;
+    o->iters = total;
+    o->cycles = cycles;
+    o->converged = s_state == 1;
+    o->nonfinite = s_state == 2 || s_nonf;
+    o->stagnated = s_state == 3;
+    o->rnorm = s_rn;
+    o->bnorm = bnorm;
   }
   leave();
 }
@@ -1443,7 +1446,7 @@ bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const
     a.pf_bytes = ((long long)(0.25 * (double)l2) / P.G) & ~15LL;
   }
   a.L = P.L;
-  reinterpret_cast<RsOut*>(c->slots_host)->pad = 1;   // the kernel's result clears it
+  reinterpret_cast<RsOut*>(c->slots_host)->timeout = 1;
   cudaError_t e;
   switch (c->precision) {
     case BIE_FP64: e = rs_launch<double, double>(P, a, c->stream); break;
@@ -1466,7 +1469,7 @@ bie_status resident_result(bie_ctx* c, bie_solve_info* info) {
   BIE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   RsOut o;
   memcpy(&o, c->slots_host, sizeof(o));
-  if (o.pad) {
+  if (o.timeout) {
     c->rs_bar = nullptr;   // cleared again before the next solve
     return ctx_fail(c, BIE_ERR_TIMEOUT, "solve: a grid barrier gave up waiting");
   }
