@@ -487,7 +487,8 @@ bie_status bie_eval_velocity(bie_ctx* ctx, const double* omega_dev, long long n,
  * Synchronises the context stream (convergence checks).  Returns
  * BIE_ERR_NOCONV if rtol was not met within max_cycles (outputs hold the last
  * iterate), BIE_ERR_NAN on a non-finite residual, BIE_ERR_TIMEOUT if a grid
- * barrier of the one-kernel solver gave up waiting (its wait is bounded). */
+ * barrier of the one-kernel solver gave up waiting (its wait is bounded); U and
+ * psi keep their values in the last two cases. */
 bie_status bie_solve(bie_ctx* ctx, const double* phit_dev, double* omega_dev, double* U_dev,
                      double* psi_dev, const bie_solve_opts* opts, bie_solve_info* info);
 

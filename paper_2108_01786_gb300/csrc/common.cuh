@@ -436,12 +436,15 @@ bie_status solve_system(bie_ctx* c, const bie_solve_opts* o, double* x, const do
                         bie_solve_info* info);
 // the solve as one cooperative kernel (resident.cu): enqueue it if it qualifies,
 // then wait for its result
-bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b, bool* taken);
+bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b, bool* taken,
+                           const unsigned** usable = nullptr);
 bie_status resident_result(bie_ctx* c, bie_solve_info* info);
 bie_status gemv_apply(bie_ctx* c, int which, const double* x_dev, double* y_dev);
 bie_status sample_run(bie_ctx* c, int which, long n, const long long* rows, const long long* cols,
                       double* out);
-bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi);
+// U and psi stay as they are where the device word *go is zero (go: may be NULL)
+bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi,
+                        const unsigned* go = nullptr);
 bie_status velocity_from_weights(bie_ctx* c, const float2* cw, const float2* hw0, double* U);
 // omega'/M_l as double-float (xh, xl: [nvec][ld], zero padded) and H omega_0'
 // (hw0: [nvec][M_0]) for nvec vectors omega ([nvec][N])

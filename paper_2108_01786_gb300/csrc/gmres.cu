@@ -1201,11 +1201,15 @@ bie_status solve_run(bie_ctx* c, const double* phit, double* omega, double* U, d
   bie_status s = rhs_run(c, phit, b);
   if (s != BIE_OK) return s;
   bool taken = false;
-  s = resident_launch(c, o, omega, b, &taken);
+  const unsigned* usable = nullptr;
+  s = resident_launch(c, o, omega, b, &taken, &usable);
   if (s != BIE_OK) return s;
-  if (taken) {   // U goes in behind the solve, one wait for both
-    s = velocity_run(c, omega, U, psi);
-    if (s != BIE_OK) return s;
+  if (taken) {   // U goes in behind the solve, one wait for both; it is left alone where the solve fails
+    s = velocity_run(c, omega, U, psi, usable);
+    if (s != BIE_OK) {   // the solve still writes the context's result slot
+      cudaStreamSynchronize(c->stream);
+      return s;
+    }
     return resident_result(c, info);
   }
   bie_status ss = (c->precision == BIE_FP64) ? run_solver<double>(c, o, omega, b, info)

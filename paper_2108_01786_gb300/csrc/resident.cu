@@ -92,7 +92,7 @@ struct RsArgs {
   void* part3;             // 2 x [row][G]
   int prow;                // rows of part1 / of one half of part3
   double* partn;           // [G]
-  unsigned* bar;           // [0] arrivals, [1] leavers; zero between solves
+  unsigned* bar;           // [0] arrivals, [1] leavers; zero between solves; [3] x is a solve's iterate
   int* err;
   unsigned spin_limit;
   RsOut* out;
@@ -579,7 +579,9 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
       __threadfence();
       if (atomicAdd(a.bar + 1, 1u) == (unsigned)G - 1) {
         __threadfence();
-        a.out->timeout = *(volatile int*)a.err;
+        const int err = *(volatile int*)a.err;
+        a.out->timeout = err;
+        a.bar[3] = !err && s_state != 2 && !s_nonf;
         a.bar[0] = 0;
         a.bar[1] = 0;
         __threadfence();
@@ -1339,8 +1341,11 @@ static cudaError_t rs_launch(const RsPlan& P, RsArgs& a, cudaStream_t st) {
 // kernel; *taken = false (and nothing enqueued) when it does not qualify: a
 // row-partitioned context (its products pass through the caller's exchange),
 // profiling (events around every product), more than RS_MAXN unknowns or a
-// restart length whose basis does not fit.  resident_result waits for it.
-bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b, bool* taken) {
+// restart length whose basis does not fit.  resident_result waits for it; *usable (may
+// be NULL) points to a device word that is zero after a solve whose x is no iterate
+// (non-finite, or a wait that ran out), for kernels enqueued behind it.
+bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const double* b, bool* taken,
+                           const unsigned** usable) {
   *taken = false;
   if (partitioned(c) || c->profiling) return BIE_OK;
   const bool ir = c->precision != BIE_FP64;
@@ -1436,6 +1441,7 @@ bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const
     if (ir) BIE_GET(c, unsigned char, "rs_U", vt * (size_t)RS_RQ * c->ld, a.Ug);
   }
   a.bar = bar;
+  if (usable) *usable = bar + 3;
   a.err = (int*)(bar + 2);
   a.spin_limit = 1u << 22;
   a.out = reinterpret_cast<RsOut*>(c->slots_dev);

@@ -178,9 +178,10 @@ __global__ void __launch_bounds__(256) k_velocity_partial(
 __global__ void k_velocity_finish(int M0, int nchunk, FlowParams F, const float2* __restrict__ part,
                                   const double2* __restrict__ z64, const double2* __restrict__ dz64,
                                   const double* __restrict__ gdiag64, const float2* __restrict__ cw,
-                                  const float2* __restrict__ hw0, double* __restrict__ U) {
+                                  const float2* __restrict__ hw0, double* __restrict__ U,
+                                  const unsigned* __restrict__ go = nullptr) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M0) return;
+  if (m >= M0 || (go && *go == 0)) return;
   dfl acc[7];
   for (int f = 0; f < 7; ++f) acc[f] = {0.f, 0.f};
   for (int ch = 0; ch < nchunk; ++ch) {
@@ -226,10 +227,11 @@ __global__ void k_velocity_finish_v(int m0, int m1, long long ld, int npanel, Fl
                                     const double* __restrict__ ypart,
                                     const double2* __restrict__ z64,
                                     const double2* __restrict__ dz64,
-                                    const float2* __restrict__ hw0, double* __restrict__ U) {
+                                    const float2* __restrict__ hw0, double* __restrict__ U,
+                                    const unsigned* __restrict__ go) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = m0 + t / OBS_SPLIT, sub = t % OBS_SPLIT;
-  if (m >= m1) return;   // whole groups leave together
+  if (m >= m1 || (go && *go == 0)) return;   // whole groups leave together
   const double2 zp = dz64[m];
   double asum = 0.0;
   for (int j = 2; j < F.nb; ++j) asum += F.a[j - 2];
@@ -242,7 +244,9 @@ __global__ void k_velocity_finish_v(int m0, int m1, long long ld, int npanel, Fl
   U[m] = (mv + y - 0.5 * h) / hypot(zp.x, zp.y);
 }
 
-__global__ void k_psi(Blocks B, const double* __restrict__ omega, double* __restrict__ psi) {
+__global__ void k_psi(Blocks B, const double* __restrict__ omega, double* __restrict__ psi,
+                      const unsigned* __restrict__ go = nullptr) {
+  if (go && *go == 0) return;
   __shared__ double red[32];
   const int k = blockIdx.x + 2;
   if (k >= B.nb) return;
@@ -327,7 +331,7 @@ bie_status velocity_from_weights(bie_ctx* c, const float2* cw, const float2* hw0
   return BIE_OK;
 }
 
-bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi) {
+bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi, const unsigned* go) {
   BIE_NVTX("normal_velocity");
   const Blocks B = make_blocks(c);
   const FlowParams F = make_flow(c);
@@ -394,14 +398,14 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi)
     const int nv = local_vrows(c);
     if (nv > 0) {
       k_velocity_finish_v<<<obs_grid(nv), NODE_THREADS, 0, c->stream>>>(c->row0, c->row0 + nv, c->ld, npanel,
-                                                                 F, ypart, z64, dz64, hw0, U);
+                                                                 F, ypart, z64, dz64, hw0, U, go);
       BIE_LAUNCH_CHECK(c, "k_velocity_finish_v");
     }
     s = part_allgather(c, U, 8, M0);   // the other parts' surface rows
     if (s != BIE_OK) return s;
     prof_end(c, pr);
     if (psi && c->nb > 2) {
-      k_psi<<<c->nb - 2, 256, 0, c->stream>>>(B, omega, psi);
+      k_psi<<<c->nb - 2, 256, 0, c->stream>>>(B, omega, psi, go);
       BIE_LAUNCH_CHECK(c, "k_psi");
     }
     return BIE_OK;
@@ -410,11 +414,11 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi)
       N, M0, nP, nQ, nPQc, z64, blk, cw, Ttab, 0.01f, part);
   BIE_LAUNCH_CHECK(c, "k_velocity_partial");
   k_velocity_finish<<<node_grid(M0), NODE_THREADS, 0, c->stream>>>(M0, nchunk, F, part, z64, dz64, gdiag64,
-                                                             cw, hw0, U);
+                                                             cw, hw0, U, go);
   prof_end(c, pr);
   BIE_LAUNCH_CHECK(c, "k_velocity_finish");
   if (psi && c->nb > 2) {
-    k_psi<<<c->nb - 2, 256, 0, c->stream>>>(B, omega, psi);
+    k_psi<<<c->nb - 2, 256, 0, c->stream>>>(B, omega, psi, go);
     BIE_LAUNCH_CHECK(c, "k_psi");
   }
   return BIE_OK;

@@ -169,3 +169,35 @@ def test_fp64_then_refined_on_one_context(P, n):
                 assert float((prob.omega - ref).norm() / ref.norm()) <= 1e-12
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_ir", "fp16_ir", "bf16_ir"])
+def test_failed_solve_leaves_U_and_psi_alone(P, prec):
+    """A non-finite right-hand side: no iterate, so U and psi keep the caller's values; a solve
+    that only missed rtol gives them from its last iterate."""
+    import torch
+    g, f, ph = _geometry(120, 61, [40, 41])
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        om = torch.empty(g.N, dtype=torch.float64, device="cuda")
+        U = torch.full((g.M[0],), 7.0, dtype=torch.float64, device="cuda")
+        psi = torch.full((2,), -3.0, dtype=torch.float64, device="cuda")
+        bad = prob.phit.clone()
+        bad[3] = float("nan")
+        for prof in (0, 1):                     # the one-kernel solver, the kernel-by-kernel one
+            P.bie_set_profiling(prob.ctx, prof)
+            with pytest.raises(P.BieError) as e:
+                P.bie_solve(prob.ctx, bad, om, U, psi)
+            assert e.value.status == P.BIE_ERR_NAN
+            assert bool((U == 7.0).all()) and bool((psi == -3.0).all()), prof
+        P.bie_set_profiling(prob.ctx, 0)
+        with pytest.raises(P.BieError) as e:
+            P.bie_solve(prob.ctx, prob.phit, om, U, psi, P.bie_default_opts(max_cycles=1, restart=2))
+        assert e.value.status == P.BIE_ERR_NOCONV
+        want = torch.empty_like(U)
+        P.bie_normal_velocity(prob.ctx, om, want)
+        assert torch.equal(U, want) and bool((psi != -3.0).all())
+        assert P.bie_solve(prob.ctx, prob.phit, om, U, psi).converged
+    finally:
+        prob.close()
