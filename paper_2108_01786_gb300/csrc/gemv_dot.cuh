@@ -3,6 +3,7 @@
 // vectors, and the double-float product-accumulate of the hi + lo residual.
 #pragma once
 #include "common.cuh"
+#include "tfl.h"
 
 template <class TA> struct Dot16;
 template <> struct Dot16<float> {
@@ -123,29 +124,16 @@ __device__ __forceinline__ dfl df_acc_prod(dfl s, float ah, float al, float xh, 
 }
 
 
-// A sum kept as three floats (about 72 bits): the flush target of short
-// double-float runs.  FP64 accumulators cost 4 FP64 instructions per flush, 64
-// cycles of an SM's FP64 pipe per warp, which is what bound the hi + lo products
-// whose matrix sits in L2; these are ~20 FP32 instructions (5 cycles).
-struct tfl {
-  float s, e, f;
-};
-__device__ __forceinline__ void tf_add(tfl& a, float h, float l) {
-  const dfl t = df_two_sum(a.s, h);
-  const dfl u = df_two_sum(a.e, l);
-  const dfl w = df_two_sum(u.hi, t.lo);
-  a.s = t.hi;
-  a.e = w.hi;
-  a.f += u.lo + w.lo;
+// Three-float sums (tfl.h) are the flush target of short double-float runs: FP64
+// accumulators cost 4 FP64 instructions per flush, 64 cycles of an SM's FP64 pipe per
+// warp, which is what bound the hi + lo products whose matrix sits in L2; these are ~20
+// FP32 instructions (5 cycles).
+__device__ __forceinline__ tfl tf_lane(tfl a, int o) {
+  return {__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.e, o),
+          __shfl_xor_sync(0xffffffffu, a.f, o)};
 }
 __device__ __forceinline__ tfl tf_warp_sum(tfl a) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float s = __shfl_xor_sync(0xffffffffu, a.s, o), e = __shfl_xor_sync(0xffffffffu, a.e, o);
-    const float f = __shfl_xor_sync(0xffffffffu, a.f, o);
-    tf_add(a, s, e);
-    a.f += f;
-  }
+  for (int o = 16; o > 0; o >>= 1) a = a + tf_lane(a, o);
   return a;
 }
-__device__ __forceinline__ double tf_to_double(tfl a) { return (double)a.s + ((double)a.e + (double)a.f); }

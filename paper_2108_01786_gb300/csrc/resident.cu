@@ -17,8 +17,7 @@
 //     inner storage (all of it up to ~3900 unknowns in 16 bits), read once;
 //   * FP64 issue: an SM retires two FP64 lanes a cycle, and adding 50 rows of
 //     152 partial sums in FP64 on every SM takes 5 us.  Partial sums are
-//     exchanged and added as double-float on the FP32 pipes (FP64 for the
-//     plain FP64 scheme, whose vectors are FP64).
+//     exchanged and added on the FP32 pipes, in two or three floats (below).
 // The Hessenberg work (a chain of ~200 dependent FP64 operations) runs on a
 // warp of its own in every CTA, from identical data, so nothing is published;
 // when a product is short (RsArgs::lag) it runs beside the next product, one
@@ -31,13 +30,14 @@
 //   D(j)   v_j, z_{j+1} of the own rows; dots of z_{j+1}
 //   UPDATE x += |r| P (Z y + U (c_0 - B y)); C and U grow
 //
-// Measured (GB300, bie_solve alone against the kernel-by-kernel solver): 640
-// unknowns FP32 646 -> 343 us, 1001 FP64 641 -> 416, 4099 BF16 873 -> 534, 16383
-// FP16 3200 -> 3054 (there HBM bounds it; what is saved is the chain between
-// products).
+// Measured (GB300, bie_solve_b back to back against the kernel-by-kernel solver): 640
+// unknowns FP32 690 -> 340 us, 1001 FP64 665 -> 364, 2944 FP16 876 -> 487, 4099 BF16 796 -> 476,
+// 8256 FP16 1344 -> 990, 16383 FP16 2697 -> 2530 (there HBM bounds it; what is saved is the
+// chain between products).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 #include "nvtx.cuh"
@@ -61,7 +61,7 @@ static_assert(sizeof(RsOut) <= sizeof(HostSlot) * BIE_NSLOTS, "result fits the s
 
 // byte offsets of the shared-memory arrays
 struct RsLayout {
-  unsigned V, C, Z, U, w, r, ry, red, xo, s1, s3, cs, sn, g, hraw, braw, hfin, rinv, H, B, c0, y, tq, Ri, Mq, RiF, MqF,
+  unsigned V, C, Z, U, w, r, ry, red, xo, s1, s3, cs, sn, g, hraw, braw, hfin, hnew, bnew, rinv, H, B, c0, y, tq, Ri, Mq, RiF, MqF,
       zmean, umean, f1, wt, A;
   unsigned total;
 };
@@ -88,9 +88,8 @@ struct RsArgs {
   float* xl;               //     and lo
   void* Zg;                // (m + 1) x ld and RS_RQ x ld: Z and U when not in shared memory
   void* Ug;
-  void* part1;             // [row][G] partial sums: float2 (FP64 scheme: float4)
-  void* part3;             // 2 x [row][G]
-  int prow;                // rows of part1 / of one half of part3
+  float4* part;            // 3 x [row][G] partial sums: of w, and two halves of z_j
+  int prow;                // rows of one of them
   double* partn;           // [G]
   unsigned* bar;           // [0] arrivals, [1] leavers; zero between solves; [3] x is a solve's iterate
   int* err;
@@ -174,79 +173,183 @@ __device__ __forceinline__ void rs_rotate2(double* hA, const double* hB, const d
 }
 
 // ---------------------------------------------------------------------------
-// partial sums: double-float for FP32 vectors, FP64 for FP64 vectors
+// Partial sums, no less accurate than the kernel-by-kernel solver's.  The dots of
+// w = A z_j and of a cycle's z_0 and the sums over obstacles, FP64 there, are three floats
+// (tfl.h, 72 bits) from the lanes' products, exact in two floats, to the sum over the
+// CTAs.  The dots of the later z_j, FP32 runs of eight added in FP64 there, are
+// double-float (48 bits).  FP64 vectors are added in FP64 within a CTA and exchanged as
+// three floats.  (FP64 throughout takes 1.5 us on every SM for 10 additions a row over
+// 20 rows, twice a step.  Double-float throughout, 5 bits short of FP64, took 342 us at
+// 640 unknowns and 461 at 4099, this 340 and 476.)
+// Three floats have FP32's exponents: |z| = 1, and |A z|^2 would have to leave 2^-96 ..
+// 2^127 for a word to be lost, where the diagonal of +-1/2 makes the system singular to
+// FP64 anyway (condition above 10^14 at the one end, 10^19 at the other).
 // ---------------------------------------------------------------------------
-template <class VT> struct RsAcc;
-template <> struct RsAcc<float> {
+template <class VT, bool F> struct RsAcc;   // F: three words exchanged, else two
+template <> struct RsAcc<float, true> {
+  typedef tfl T;           // a lane's sum
+  typedef tfl X;           // as exchanged and added over the CTAs
+  typedef float4 S;        // a sum over the CTAs: its nearest float first, unused last
+  static constexpr int LD = 5;   // exchanged values in flight per lane
+  static __device__ __forceinline__ T zero() { return {0.f, 0.f, 0.f}; }
+  static __device__ __forceinline__ T mad(T s, float a, float b) {
+    const dfl p = df_two_prod(a, b);
+    tf_add(s, p.hi, p.lo);
+    return s;
+  }
+  static __device__ __forceinline__ T addv(T s, float a) {
+    tf_add(s, a, 0.f);
+    return s;
+  }
+  static __device__ __forceinline__ T warp(T a) { return tf_warp_sum(a); }
+  static __device__ __forceinline__ X split(T a) { return a; }
+  static __device__ __forceinline__ S pack(X a) {
+    a = tf_norm(a);
+    return make_float4(a.s, a.e, a.f, 0.f);
+  }
+};
+template <> struct RsAcc<float, false> {
   typedef dfl T;
-  typedef float2 S;        // as stored
-  typedef float2 X;        // as exchanged
-  typedef dfl XT;          // as added over the CTAs
-  static constexpr int LD = 10;   // exchanged values in flight per lane (16 lanes: 160 CTAs)
-  static __device__ __forceinline__ X xpack(T a) { return make_float2(a.hi, a.lo); }
-  static __device__ __forceinline__ XT xzero() { return {0.f, 0.f}; }
-  static __device__ __forceinline__ void xadd(XT& s, X v) { s = s + dfl{v.x, v.y}; }
-  static __device__ __forceinline__ void xadd_lane(XT& s, int o) { s = s + shfl(s, o); }
-  static __device__ __forceinline__ S xout(XT a) { return make_float2(a.hi, a.lo); }
+  typedef dfl X;
+  typedef float4 S;
+  static constexpr int LD = 10;
   static __device__ __forceinline__ T zero() { return {0.f, 0.f}; }
   static __device__ __forceinline__ T mad(T s, float a, float b) {
     const dfl p = df_two_prod(a, b);
     const dfl t = df_two_sum(s.hi, p.hi);
     return df_fast_two_sum(t.hi, t.lo + (s.lo + p.lo));
   }
-  static __device__ __forceinline__ T addv(T s, float a) { return df_addf(s, a); }
-  static __device__ __forceinline__ S pack(T a) { return make_float2(a.hi, a.lo); }
-  static __device__ __forceinline__ T unpack(S a) { return {a.x, a.y}; }
-  static __device__ __forceinline__ double value(T a) { return (double)a.hi + (double)a.lo; }
-  static __device__ __forceinline__ float head(T a) { return a.hi; }
-  // 1 / sqrt(a) (0 for a <= 0): one Newton step from the FP32 value
-  static __device__ __forceinline__ T rsqrt_pos(T a) {
-    if (!(a.hi > 0.f)) return zero();
-    const float x = rsqrtf(a.hi);
-    const dfl e = dfl{1.f, 0.f} - a * df_two_prod(x, x);
-    return df_fast_two_sum(x, 0.5f * x * e.hi);
-  }
-  static __device__ __forceinline__ T shfl(T a, int o) {
-    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
-  }
+  static __device__ __forceinline__ T warp(T a) { return warp_sum(a); }
+  static __device__ __forceinline__ X split(T a) { return a; }
+  static __device__ __forceinline__ S pack(X a) { return make_float4(a.hi, a.lo, 0.f, 0.f); }
 };
-// (FP64 vectors: sums within a CTA in FP64, exchanged as three floats, which hold
-// an FP64 value, and added over the CTAs as such: on every SM 10 FP64 additions a
-// row over 20 rows are 1.5 us, twice a step)
-template <> struct RsAcc<double> {
+template <> struct RsAcc<double, true> {
   typedef double T;
+  typedef tfl X;
   typedef double S;
-  typedef float4 X;
-  typedef tfl XT;
   static constexpr int LD = 5;
-  static __device__ __forceinline__ X xpack(T a) {
-    const float h = (float)a;
-    const double r = a - (double)h;
-    const float l = (float)r;
-    return make_float4(h, l, (float)(r - (double)l), 0.f);
-  }
-  static __device__ __forceinline__ XT xzero() { return {0.f, 0.f, 0.f}; }
-  static __device__ __forceinline__ void xadd(XT& s, X v) {
-    tf_add(s, v.x, v.y);
-    s.f += v.z;
-  }
-  static __device__ __forceinline__ void xadd_lane(XT& s, int o) {
-    const float h = __shfl_xor_sync(0xffffffffu, s.s, o), l = __shfl_xor_sync(0xffffffffu, s.e, o);
-    const float f = __shfl_xor_sync(0xffffffffu, s.f, o);
-    tf_add(s, h, l);
-    s.f += f;
-  }
-  static __device__ __forceinline__ S xout(XT a) { return tf_to_double(a); }
   static __device__ __forceinline__ T zero() { return 0.0; }
   static __device__ __forceinline__ T mad(T s, double a, double b) { return fma(a, b, s); }
   static __device__ __forceinline__ T addv(T s, double a) { return s + a; }
-  static __device__ __forceinline__ S pack(T a) { return a; }
-  static __device__ __forceinline__ T unpack(S a) { return a; }
-  static __device__ __forceinline__ double value(T a) { return a; }
-  static __device__ __forceinline__ double head(T a) { return a; }
-  static __device__ __forceinline__ T rsqrt_pos(T a) { return a > 0.0 ? rs_rsqrt(a) : 0.0; }
-  static __device__ __forceinline__ T shfl(T a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+  static __device__ __forceinline__ T warp(T a) { return warp_sum(a); }
+  static __device__ __forceinline__ X split(T a) {
+    const float h = (float)a;
+    const double r = a - (double)h;
+    const float l = (float)r;
+    return {h, l, (float)(r - (double)l)};
+  }
+  static __device__ __forceinline__ S pack(X a) { return tf_to_double(a); }
 };
+
+// Exchange: value i (row r of CTA c at i = r G + c) of a region, 16 bytes as three words or 8
+// as two.  The rows of one region in two words come before those in three.
+__device__ __forceinline__ void rs_put(float4* p, size_t i, tfl v) { p[i] = make_float4(v.s, v.e, v.f, 0.f); }
+__device__ __forceinline__ void rs_put(float4* p, size_t i, dfl v) {
+  reinterpret_cast<float2*>(p)[i] = make_float2(v.hi, v.lo);
+}
+__device__ __forceinline__ void rs_get(const float4* p, size_t i, tfl& v) {
+  const float4 a = __ldcg(p + i);
+  v = {a.x, a.y, a.z};
+}
+__device__ __forceinline__ void rs_get(const float4* p, size_t i, dfl& v) {
+  const float2 a = __ldcg(reinterpret_cast<const float2*>(p) + i);
+  v = {a.x, a.y};
+}
+__device__ __forceinline__ void rs_zero(tfl& v) { v = {0.f, 0.f, 0.f}; }
+__device__ __forceinline__ void rs_zero(dfl& v) { v = {0.f, 0.f}; }
+__device__ __forceinline__ void rs_zero(double& v) { v = 0.0; }
+__device__ __forceinline__ tfl rs_lane(tfl s, int o) { return tf_lane(s, o); }
+__device__ __forceinline__ dfl rs_lane(dfl s, int o) {
+  return {__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
+}
+__device__ __forceinline__ double rs_lane(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+// a sum over the CTAs: its value, and its head in the vectors' type
+__device__ __forceinline__ double rs_value(const float4& a) { return tf_to_double({a.x, a.y, a.z}); }
+__device__ __forceinline__ double rs_value(double a) { return a; }
+__device__ __forceinline__ float rs_head(const float4& a) { return a.x; }
+__device__ __forceinline__ float rs_head(dfl a) { return a.hi; }
+__device__ __forceinline__ double rs_head(double a) { return a; }
+
+// What follows from the sums (nu, h_j, beta) is ~35 dependent operations: 2400 cycles in
+// double-float, 4100 in three floats, 6600 in FP64 beside other FP64 work.  The Hessenberg
+// matrix takes the three-float values, formed by three warps beside the row work; the rows
+// take the double-float ones (43 bits and more), rounded to their own FP32.
+__device__ __forceinline__ void rs_sc(const float4& a, dfl& v) { v = {a.x, a.y}; }
+__device__ __forceinline__ void rs_sc(const float4& a, tfl& v) { v = {a.x, a.y, a.z}; }
+__device__ __forceinline__ void rs_sc(double a, double& v) { v = a; }
+// 1 / sqrt(a), 0 for a <= 0
+__device__ __forceinline__ dfl rs_rsqrt_pos(dfl a) {   // one Newton step from the FP32 value
+  if (!(a.hi > 0.f)) return {0.f, 0.f};
+  const float x = rsqrtf(a.hi);
+  const dfl e = dfl{1.f, 0.f} - a * df_two_prod(x, x);
+  return df_fast_two_sum(x, 0.5f * x * e.hi);
+}
+__device__ __forceinline__ double rs_rsqrt_pos(double a) { return a > 0.0 ? rs_rsqrt(a) : 0.0; }
+__device__ __forceinline__ tfl rs_rsqrt_pos(tfl a) { return tf_rsqrt_from(a, rsqrtf(a.s)); }
+
+template <class VT> struct RsHead { typedef dfl T; };   // what the rows' scalars are formed in
+template <> struct RsHead<double> { typedef double T; };
+// sum_i a_i b_i, i < n, by one warp (every lane gets it)
+template <class T, class S>
+__device__ __forceinline__ T rs_sum(const S* a, const S* b, int n) {
+  T t;
+  rs_zero(t);
+  for (int i = threadIdx.x & 31; i < n; i += 32) {
+    T u, v;
+    rs_sc(a[i], u);
+    rs_sc(b[i], v);
+    t = t + u * v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t = t + rs_lane(t, o);
+  return t;
+}
+template <class T> struct RsScal {
+  T nu, inu, hj, beta, ibe;
+};
+// nu, h_j, beta of a step (see k_dcgs) by one warp; s3, s1: the sums of z_j and of w
+template <class T, class S>
+__device__ __forceinline__ RsScal<T> rs_scalars(const S* s3, const S* s1, int nb) {
+  T ta, tas, tss;
+  rs_zero(ta);
+  rs_zero(tas);
+  rs_zero(tss);
+  for (int i = threadIdx.x & 31; i < nb; i += 32) {
+    T v3, v1;
+    rs_sc(s3[i], v3);
+    rs_sc(s1[i], v1);
+    ta = ta + v3 * v3;
+    tas = tas + v3 * v1;
+    tss = tss + v1 * v1;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ta = ta + rs_lane(ta, o);
+    tas = tas + rs_lane(tas, o);
+    tss = tss + rs_lane(tss, o);
+  }
+  T a, sg, om;
+  rs_sc(s3[nb], a);
+  rs_sc(s1[nb], sg);
+  rs_sc(s1[nb + 1], om);
+  RsScal<T> r;
+  const T nu2 = a - ta;
+  r.inu = rs_rsqrt_pos(nu2);
+  r.nu = nu2 * r.inu;
+  r.hj = (sg - tas) * r.inu;
+  const T be2 = om - tss - r.hj * r.hj;
+  r.ibe = rs_rsqrt_pos(be2);
+  r.beta = be2 * r.ibe;
+  return r;
+}
+
+// coef a im rounded to FP32 (a few 2^-48 more): an obstacle's share of the preconditioner
+// from its sum a
+__device__ __forceinline__ float rs_share(const float4& a, float im, float coef) {
+  const dfl p = df_two_prod(a.x, im);
+  return fmaf(coef, p.hi, coef * fmaf(a.y, im, p.lo));
+}
+__device__ __forceinline__ double rs_share(double a, double im, double coef) { return coef * (a * im); }
 
 // ---------------------------------------------------------------------------
 // grid barrier: arrivals counted upward through the solve (epoch e waits for
@@ -282,41 +385,52 @@ __device__ __forceinline__ void rs_bar_rows(int n) {   // the row warps only
   asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory");
 }
 
-// Sums over the G CTAs of the rows of `part`: 16 lanes per row, fixed order.  The
-// first rows' loads are issued by rs_load so that other work can hide them;
-// rs_reduce adds them and takes the remaining rows (nthr threads take part).
-template <class VT>
-__device__ __forceinline__ void rs_load(const typename RsAcc<VT>::X* part, int cnt, int G,
-                                        typename RsAcc<VT>::X* v, int base = 0) {
-  typedef RsAcc<VT> AC;
-  const int i = base + (int)(threadIdx.x >> 4), q = threadIdx.x & 15;
+// the scalars of a step: ready (not waiting), and waited for by the Hessenberg warp
+__device__ __forceinline__ void rs_arrive_scal(int n) {
+  __syncwarp();
+  asm volatile("bar.arrive 3, %0;" ::"r"(n) : "memory");
+}
+__device__ __forceinline__ void rs_bar_scal(int n) {
+  asm volatile("bar.sync 3, %0;" ::"r"(n) : "memory");
+}
+
+// Sums over the G CTAs of the rows of `part`, fixed order, LN lanes per row: 16, or 32 where
+// the loads in flight of 16 lanes would not cover the CTAs (a second round of loads costs
+// as much as the first: 4099 unknowns 510 -> 487 us).  The first rows' loads are issued by
+// rs_load so that other work can hide them; rs_reduce adds them and takes the remaining
+// rows (nthr threads take part).
+template <class AC, int LN>
+__device__ __forceinline__ void rs_load(const float4* part, int cnt, int G, typename AC::X* v, int base = 0) {
+  const int i = base + (int)threadIdx.x / LN, q = threadIdx.x % LN;
 #pragma unroll
   for (int u = 0; u < AC::LD; ++u) {
-    const int c = q + 16 * u;
-    if (i < cnt && c < G) v[u] = __ldcg(part + (size_t)i * G + c);
-    else v[u] = AC::xpack(AC::zero());
+    const int c = q + LN * u;
+    rs_zero(v[u]);
+    if (i < cnt && c < G) rs_get(part, (size_t)i * G + c, v[u]);
   }
 }
-template <class VT>
-__device__ __forceinline__ void rs_reduce(const typename RsAcc<VT>::X* part, int cnt, int G,
-                                          typename RsAcc<VT>::X* v, typename RsAcc<VT>::S* out, int nthr) {
-  typedef RsAcc<VT> AC;
-  const int q = threadIdx.x & 15;
-  for (int base = 0; base < cnt; base += nthr >> 4) {
-    const int i = base + (int)(threadIdx.x >> 4);
-    if (base > 0) rs_load<VT>(part, cnt, G, v, base);
-    typename AC::XT s = AC::xzero();
+template <class AC, int LN>
+__device__ __forceinline__ void rs_reduce(const float4* part, int cnt, int G, typename AC::X* v,
+                                          typename AC::S* out, int nthr) {
+  const int q = threadIdx.x % LN;
+  for (int base = 0; base < cnt; base += nthr / LN) {
+    const int i = base + (int)threadIdx.x / LN;
+    if (base > 0) rs_load<AC, LN>(part, cnt, G, v, base);
+    typename AC::X s = v[0];
 #pragma unroll
-    for (int u = 0; u < AC::LD; ++u)
-      if (16 * u < G) AC::xadd(s, v[u]);
+    for (int u = 1; u < AC::LD; ++u)
+      if (LN * u < G) s = s + v[u];
     if (i < cnt) {
-#pragma unroll 5
-      for (int c = q + 16 * AC::LD; c < G; c += 16) AC::xadd(s, __ldcg(part + (size_t)i * G + c));
+      for (int c = q + LN * AC::LD; c < G; c += LN) {
+        typename AC::X t;
+        rs_get(part, (size_t)i * G + c, t);
+        s = s + t;
+      }
     }
     __syncwarp();
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) AC::xadd_lane(s, o);
-    if (i < cnt && q == 0) out[i] = AC::xout(s);
+    for (int o = LN / 2; o > 0; o >>= 1) s = s + rs_lane(s, o);
+    if (i < cnt && q == 0) out[i] = AC::pack(s);
   }
 }
 
@@ -494,7 +608,8 @@ __device__ __forceinline__ void rs_stage(T* dst, const void* src, long long n, i
 template <class TA, class VT>
 __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ RsArgs a) {
   constexpr bool RC = sizeof(VT) == 4;      // refined scheme: recycled space, hi + lo residuals
-  typedef RsAcc<VT> AC;
+  typedef RsAcc<VT, true> AC;        // dots of w and of z_0
+  typedef RsAcc<VT, !RC> AZ;         // dots of the later z_j
   extern __shared__ __align__(16) unsigned char sm[];
   VT* xs = reinterpret_cast<VT*>(sm);       // 8 ld bytes: x (FP64), or hi and lo
   const RsLayout& L = a.L;
@@ -504,7 +619,6 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
   double* sr = reinterpret_cast<double*>(sm + L.r);
   double* sx = reinterpret_cast<double*>(sm + L.xo);   // x, then the last increment (2 x R)
   typedef typename AC::S PS;
-  typedef typename AC::X PX;
   typedef typename AC::T PT;
   PS* s1 = reinterpret_cast<PS*>(sm + L.s1);           // reduced dots of w
   PS* s3 = reinterpret_cast<PS*>(sm + L.s3);           // reduced dots of z_j, 2 halves
@@ -516,6 +630,8 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
   double* h_raw = reinterpret_cast<double*>(sm + L.hraw);
   double* h_braw = reinterpret_cast<double*>(sm + L.braw);
   double* h_fin = reinterpret_cast<double*>(sm + L.hfin);   // a Hessenberg column being finished
+  double* h_new = reinterpret_cast<double*>(sm + L.hnew);    // the provisional column, not yet accepted
+  double* h_bnew = reinterpret_cast<double*>(sm + L.bnew);
   double* h_rinv = reinterpret_cast<double*>(sm + L.rinv);  // 1 / R_ii
   double* Hm = reinterpret_cast<double*>(sm + L.H);    // column c at c (c + 1) / 2
   double* Bm = reinterpret_cast<double*>(sm + L.B);    // column c at c RS_RQ
@@ -532,12 +648,14 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
   VT* swt = reinterpret_cast<VT*>(sm + L.wt);                // 1 / M, diagonal and row flip of the own rows (3 x R)
   uint4* sA = reinterpret_cast<uint4*>(sm + L.A);            // kv vectors of every own row
   __shared__ int s_ok, s_done, s_iters, s_nonf, s_state, s_kd, s_kn, s_lost;
+  __shared__ double s_bprev, s_ua, s_ub;   // the Hessenberg warp's, between its two parts
   __shared__ double s_gpre, s_rn, s_inv, s_tol, s_red[4];
-  __shared__ PT s_nu, s_hj, s_beta;
+  __shared__ double s_nu, s_hj, s_beta;
+  __shared__ tfl s_less[2];                // z_j^T w and |w|^2 less their parts in [C, V]
   __shared__ VT s_c, s_s;
   __shared__ VT s_xc[BIE_MAXB];
   __shared__ double s_dm[BIE_MAXB];
-  __shared__ VT s_inu, s_ib;
+  __shared__ VT s_inu, s_ib, s_vh;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nw = blockDim.x >> 5, nrw = nw - 1, nrt = 32 * nrw;
@@ -551,8 +669,8 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
   const size_t zst = a.zsm ? (size_t)R : (size_t)ld;         // stride of Z and U columns
   VT* zb = reinterpret_cast<VT*>(a.zbuf);
   const size_t phalf = (size_t)a.prow * G;
-  PX* part1 = reinterpret_cast<PX*>(a.part1);
-  PX* part3[2] = {reinterpret_cast<PX*>(a.part3), reinterpret_cast<PX*>(a.part3) + phalf};
+  float4* const part1 = a.part;             // partial sums of w; then two halves of those of z_j
+  auto part3 = [&](int h) -> float4* { return a.part + (h + 1) * phalf; };
   constexpr int E = 16 / (int)sizeof(TA);
   const int nvec = (int)(ld / E), kv = a.kv;
   const uint4* A = reinterpret_cast<const uint4*>(a.A) + (size_t)c0r * nvec;
@@ -798,46 +916,60 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
         const int a0 = max(0, a.obs_off[k] - c0r), a1 = min(nr, a.obs_off[k + 1] - c0r);
         for (int t = a0 + lane; t < a1; t += 32) s = AC::addv(s, V[t]);
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s = s + AC::shfl(s, o);
-      if (lane == 0) part3[0][(size_t)i * G + blockIdx.x] = AC::xpack(s);
+      s = AC::warp(s);
+      if (lane == 0) rs_put(part3(0), (size_t)i * G + blockIdx.x, AC::split(s));
     }
     if (!rs_barrier(a, epoch, &s_ok)) { leave(); return; }
 
-    // Hessenberg columns j - 1 (final) and j (provisional), rotations, test; by
-    // the Hessenberg warp (see k_dcgs for the derivation)
-    auto hwork = [&](int j, bool lost, bool brk) {
+    // Hessenberg columns j - 1 (final) and j (provisional), rotations, test; by the
+    // Hessenberg warp (see k_dcgs for the derivation).  First what the sums alone give ...
+    auto hcolumns = [&](int j) {
       const PS* S3 = s3 + (size_t)(j & 1) * s3n;
-      auto v1 = [&](int i) -> double { return AC::value(AC::unpack(s1[i])); };
-      auto v3 = [&](int i) -> double { return AC::value(AC::unpack(S3[i])); };
-      const double nu = AC::value(s_nu), hj = AC::value(s_hj), beta = AC::value(s_beta);
+      auto v1 = [&](int i) -> double { return rs_value(s1[i]); };
+      auto v3 = [&](int i) -> double { return rs_value(S3[i]); };
       for (int o = lane; o < nobs; o += 32)   // means of z_j over the obstacles
         zmean[(size_t)j * nobs + o] = v3(q + j + 1 + o) * (double)a.obs_invM[o];
       // column j - 1 is final: h + bprev a', subdiagonal bprev nu
       const double bprev = j > 0 ? h_raw[j] : 0.0;
-      for (int i = lane; i < j; i += 32) h_fin[i] = fma(bprev, v3(q + i), h_raw[i]);
-      if (j > 0)
-        for (int i = lane; i < q; i += 32) Bm[(size_t)(j - 1) * RS_RQ + i] = fma(bprev, v3(i), h_braw[i]);
-      else
-        for (int i = lane; i < q; i += 32) c0[i] = v3(i);
+      for (int i = lane; i < j; i += 32) {
+        h_fin[i] = fma(bprev, v3(q + i), h_raw[i]);
+        h_new[i] = v1(q + i);
+      }
+      for (int i = lane; i < q; i += 32) {
+        if (j > 0) Bm[(size_t)(j - 1) * RS_RQ + i] = fma(bprev, v3(i), h_braw[i]);
+        else c0[i] = v3(i);
+        h_bnew[i] = v1(i);
+      }
       __syncwarp();
-      if (!lost) {   // the provisional column j replaces it as the last raw one
-        for (int i = lane; i < j; i += 32) h_raw[i] = v1(q + i);
-        for (int i = lane; i < q; i += 32) h_braw[i] = v1(i);
+      if (j > 0) {
+        double ua, ub;
+        rs_rotate2(h_fin, h_new, h_cs, h_sn, j - 1, ua, ub);
+        if (lane == 0) {
+          s_bprev = bprev;
+          s_ua = ua;
+          s_ub = ub;
+        }
+      }
+      __syncwarp();
+    };
+    // ... then what takes nu, h_j and beta
+    auto hfinish = [&](int j, bool lost, bool brk) {
+      const double nu = s_nu, hj = s_hj, beta = s_beta;
+      if (!lost) {   // the provisional column j replaces column j - 1 as the last raw one
+        for (int i = lane; i < j; i += 32) h_raw[i] = h_new[i];
+        for (int i = lane; i < q; i += 32) h_braw[i] = h_bnew[i];
         if (lane == 0) {
           h_raw[j] = hj;
           h_raw[j + 1] = beta;
         }
       }
-      __syncwarp();
       double gj = nu, uj = hj;   // z_0 = C c_0 + nu v_0: the right-hand side in H is nu e_1
       if (j > 0) {
-        double ua, ub, c, s, rr, ir;
-        rs_rotate2(h_fin, h_raw, h_cs, h_sn, j - 1, ua, ub);
-        rs_givens(ua, bprev * nu, c, s, rr, ir);
+        double c, s, rr, ir;
+        rs_givens(s_ua, s_bprev * nu, c, s, rr, ir);
         const double gpre = s_gpre;
         gj = -s * gpre;
-        uj = fma(-s, ub, c * hj);
+        uj = fma(-s, s_ub, c * hj);
         __syncwarp();
         if (lane == 0) {
           h_cs[j - 1] = c;
@@ -876,20 +1008,66 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
       const bool lagged = a.lag && j > 0;
       // G(j)
       if (!hwarp) {
-        PX ld3[AC::LD];   // the dots of z_j reduce while it is staged
         const int n3 = nb + 1 + nobs;
         PS* S3 = s3 + (size_t)(j & 1) * s3n;
-        rs_load<VT>(part3[j & 1], n3, G, ld3);
-        rs_stage<VT>(xs, zb, ld, nrt);
-        rs_reduce<VT>(part3[j & 1], n3, G, ld3, S3, nrt);
+        auto take = [&](auto acc) {   // the dots of z_j reduce while it is staged
+          typedef decltype(acc) A3;
+          constexpr bool all = std::is_same<A3, AC>::value;   // the sums over obstacles too
+          constexpr int LN = RC ? 16 : 32;
+          const int nd = all ? n3 : nb + 1;
+          typename A3::X ld3[A3::LD];
+          // an obstacle's sum (three words) goes to a warp that has none of the first rows
+          const int ob = nrw - 1 - warp;
+          const bool mine = !all && ob < nobs && 2 * warp >= nd && nd <= nrt / LN && G <= 32 * A3::LD / 2;
+          if constexpr (!all) {
+            if (mine) {
+#pragma unroll
+              for (int u = 0; u < A3::LD / 2; ++u) {
+                tfl v = {0.f, 0.f, 0.f};
+                if (lane + 32 * u < G) rs_get(part3(j & 1), (size_t)(nb + 1 + ob) * G + lane + 32 * u, v);
+                ld3[2 * u] = {v.s, v.e};
+                ld3[2 * u + 1] = {v.f, 0.f};
+              }
+            } else {
+              rs_load<A3, LN>(part3(j & 1), nd, G, ld3);
+            }
+          } else {
+            rs_load<A3, LN>(part3(j & 1), nd, G, ld3);
+          }
+          rs_stage<VT>(xs, zb, ld, nrt);
+          if constexpr (!all) {
+            if (mine) {
+              tfl s = {ld3[0].hi, ld3[0].lo, ld3[1].hi};
+#pragma unroll
+              for (int u = 1; u < A3::LD / 2; ++u) s = s + tfl{ld3[2 * u].hi, ld3[2 * u].lo, ld3[2 * u + 1].hi};
+              s = tf_warp_sum(s);
+              if (lane == 0) S3[nb + 1 + ob] = AC::pack(s);
+            } else {
+              rs_reduce<A3, LN>(part3(j & 1), nd, G, ld3, S3, nrt);
+              for (int o = ob; o < nobs; o += nrw) {
+                tfl s = {0.f, 0.f, 0.f};
+                for (int c = lane; c < G; c += 32) {
+                  tfl v;
+                  rs_get(part3(j & 1), (size_t)(nb + 1 + o) * G + c, v);
+                  s = s + v;
+                }
+                s = tf_warp_sum(s);
+                if (lane == 0) S3[nb + 1 + o] = AC::pack(s);
+              }
+            }
+          } else {
+            rs_reduce<A3, LN>(part3(j & 1), nd, G, ld3, S3, nrt);
+          }
+        };
+        if (j == 0) take(AC());
+        else take(AZ());
         rs_bar_rows(nrt);
         if (nobs > 0) {   // P z_j: each obstacle's entries lower by coef mean / M
           if ((int)threadIdx.x < nobs)
-            s_xc[threadIdx.x] = (VT)a.obs_coef * (AC::head(AC::unpack(S3[nb + 1 + threadIdx.x])) *
-                                                  (VT)a.obs_invM[threadIdx.x]);
+            s_xc[threadIdx.x] = rs_share(S3[nb + 1 + threadIdx.x], a.obs_invM[threadIdx.x], a.obs_coef);
           for (int o = 0; o < nobs; ++o) {
             const VT im = (VT)a.obs_invM[o];
-            const VT cw = (VT)a.obs_coef * (AC::head(AC::unpack(S3[nb + 1 + o])) * im) * im;
+            const VT cw = rs_share(S3[nb + 1 + o], im, a.obs_coef) * im;
             for (int c = a.obs_off[o] + (int)threadIdx.x; c < a.obs_off[o + 1]; c += nrt) xs[c] -= cw;
           }
           rs_bar_rows(nrt);
@@ -922,12 +1100,12 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
           const VT* qi = i <= nb ? qv(q, i) : sw;
           PT s = AC::zero();
           for (int t = lane; t < nr; t += 32) s = AC::mad(s, qi[t], sw[t]);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) s = s + AC::shfl(s, o);
-          if (lane == 0) part1[(size_t)i * G + blockIdx.x] = AC::xpack(s);
+          s = AC::warp(s);
+          if (lane == 0) rs_put(part1, (size_t)i * G + blockIdx.x, AC::split(s));
         }
       } else if (lagged) {
-        hwork(j - 1, false, false);
+        hcolumns(j - 1);
+        hfinish(j - 1, false, false);
       }
       if (!rs_barrier(a, epoch, &s_ok)) { leave(); return; }
       if (lagged && s_done) {   // the previous step ended the cycle; this product is dropped
@@ -944,92 +1122,128 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
         }
       }
       {
-        PX ld1[AC::LD];
-        rs_load<VT>(part1, nb + 2, G, ld1);
-        rs_reduce<VT>(part1, nb + 2, G, ld1, s1, blockDim.x);
+        typename AC::X ld1[AC::LD];
+        if (G > 16 * AC::LD) {
+          rs_load<AC, 32>(part1, nb + 2, G, ld1);
+          rs_reduce<AC, 32>(part1, nb + 2, G, ld1, s1, blockDim.x);
+        } else {
+          rs_load<AC, 16>(part1, nb + 2, G, ld1);
+          rs_reduce<AC, 16>(part1, nb + 2, G, ld1, s1, blockDim.x);
+        }
       }
       __syncthreads();
       const PS* S3 = s3 + (size_t)(j & 1) * s3n;
-      if (warp == 0) {   // nu, h_j, beta (see k_dcgs), in the partial sums' arithmetic
-        PT ta = AC::zero(), tas = AC::zero(), tss = AC::zero();
-        for (int i = lane; i < nb; i += 32) {
-          const PT v3 = AC::unpack(S3[i]), v1 = AC::unpack(s1[i]);
-          ta = ta + v3 * v3;
-          tas = tas + v3 * v1;
-          tss = tss + v1 * v1;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          ta = ta + AC::shfl(ta, o);
-          tas = tas + AC::shfl(tas, o);
-          tss = tss + AC::shfl(tss, o);
-        }
-        if (lane == 0) {
-          const PT nu2 = AC::unpack(S3[nb]) - ta;
-          const PT inu = AC::rsqrt_pos(nu2);
-          const PT nu = nu2 * inu;
-          const VT nuh = AC::head(nu);
-          const PT hj = (AC::unpack(s1[nb]) - tas) * inu;
-          const PT be2 = AC::unpack(s1[nb + 1]) - tss - hj * hj;
-          const PT ibe = AC::rsqrt_pos(be2);
-          const PT beta = be2 * ibe;
-          const VT bh = AC::head(beta);
-          // z_j lies in span [C, V] (to rounding): column j - 1 is the cycle's last one
-          const bool lost = !(nuh > (VT)0) || !isfinite(nuh) || !isfinite(AC::head(hj));
-          const bool brk = lost || !(bh > (VT)0) || !isfinite(bh);
-          s_nu = nu;
-          s_hj = hj;
-          s_beta = beta;
-          s_inu = AC::head(inu);
-          s_ib = brk ? (VT)0 : AC::head(ibe);
-          s_lost = lost ? 2 : brk ? 1 : 0;
-        }
-      }
-      __syncthreads();
-      const bool lost = s_lost == 2, brk = s_lost != 0;
-      const bool now = !a.lag || brk || j + 1 >= m;   // the test is made in this phase
+      // The row warps subtract the basis from z_j (into vn, free until z_{j+1} goes there) and
+      // from w, while one warp forms the scalars the rows take, three the Hessenberg
+      // column's (FP64 vectors: the same ones) and the Hessenberg warp the columns
+      VT* vj = V + (size_t)j * R;
+      VT* vn = V + (size_t)(j + 1) * R;
+      const int nrow_w = RC ? nrw - 3 : nrw;          // row warps here, the last of them for the scalars
       if (hwarp) {
-        if (now) hwork(j, lost, brk);
-      } else if (!lost) {
-        const VT inu = s_inu, ib = s_ib, vh = AC::head(s_hj);
-        VT* vj = V + (size_t)j * R;
-        VT* vn = V + (size_t)(j + 1) * R;
-        for (int t = threadIdx.x; t < nr; t += nrt) {
-          VT tv = vj[t], u = sw[t];
-#pragma unroll 4
-          for (int i = 0; i < nb; ++i) {
-            const VT v = qv(q, i)[t];
-            tv -= AC::head(AC::unpack(S3[i])) * v;
-            u -= AC::head(AC::unpack(s1[i])) * v;
-          }
-          const VT vt = tv * inu;
-          vj[t] = vt;
-          const VT zz = brk ? (VT)0 : (u - vh * vt) * ib;
-          vn[t] = zz;
-          Z[(size_t)(j + 1) * zst + t] = zz;
-          zb[c0r + t] = zz * swt[t];
+        if (!a.lag) hcolumns(j);
+        rs_bar_scal(RC ? 96 : 64);
+        const bool lost = s_lost == 2, brk = s_lost != 0;
+        if (!a.lag || brk || j + 1 >= m) {            // the test is made in this phase
+          if (a.lag) hcolumns(j);
+          hfinish(j, lost, brk);
         }
-        rs_bar_rows(nrt);
-        // a' = Q_i^T z_{j+1} (i <= nb, v_j included), |z_{j+1}|^2, obstacle sums
-        PX* p3 = part3[(j + 1) & 1];
-        const int nrow = nb + 2 + nobs;
-        for (int i = warp; i < nrow; i += nrw) {
-          PT s = AC::zero();
-          if (i <= nb + 1) {
-            const VT* qi = qv(q, i);
-            for (int t = lane; t < nr; t += 32) s = AC::mad(s, qi[t], vn[t]);
+      } else if (warp >= nrow_w) {                    // RC: the Hessenberg column's scalars, a sum each
+        if constexpr (RC) {
+          tfl v;
+          if (warp == nrow_w) {
+            rs_sc(S3[nb], v);
+            const tfl nu2 = v - rs_sum<tfl>(S3, S3, nb);
+            const tfl inu = rs_rsqrt_pos(nu2);
+            const double nu = tf_to_double(nu2 * inu);
+            asm volatile("bar.sync 4, 96;" ::: "memory");
+            const tfl hj = s_less[0] * inu;
+            const tfl be2 = s_less[1] - hj * hj;
+            const double beta = tf_to_double(be2 * rs_rsqrt_pos(be2));
+            if (lane == 0) {
+              s_nu = nu;
+              s_hj = tf_to_double(hj);
+              s_beta = beta;
+            }
+            rs_arrive_scal(96);
           } else {
-            const int o = i - (nb + 2);
-            const int a0 = max(0, a.obs_off[o] - c0r), a1 = min(nr, a.obs_off[o + 1] - c0r);
-            for (int t = a0 + lane; t < a1; t += 32) s = AC::addv(s, vn[t]);
+            const bool sg = warp == nrow_w + 1;
+            rs_sc(s1[sg ? nb : nb + 1], v);
+            v = v - rs_sum<tfl>(sg ? S3 : s1, s1, nb);
+            if (lane == 0) s_less[sg ? 0 : 1] = v;
+            __syncwarp();
+            asm volatile("bar.arrive 4, 96;" ::: "memory");
           }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) s = s + AC::shfl(s, o);
-          if (lane == 0) p3[(size_t)i * G + blockIdx.x] = AC::xpack(s);
+        }
+      } else {
+        if (warp == nrow_w - 1) {
+          typedef typename RsHead<VT>::T T;
+          const RsScal<T> r = rs_scalars<T>(S3, s1, nb);
+          if (lane == 0) {
+            const VT nuh = rs_head(r.nu), bh = rs_head(r.beta), vh = rs_head(r.hj);
+            // z_j lies in span [C, V] (to rounding): column j - 1 is the cycle's last one
+            const bool lost = !(nuh > (VT)0) || !isfinite(nuh) || !isfinite(vh);
+            const bool brk = lost || !(bh > (VT)0) || !isfinite(bh);
+            if constexpr (!RC) {
+              s_nu = r.nu;
+              s_hj = r.hj;
+              s_beta = r.beta;
+            }
+            s_vh = vh;
+            s_inu = rs_head(r.inu);
+            s_ib = brk ? (VT)0 : rs_head(r.ibe);
+            s_lost = lost ? 2 : brk ? 1 : 0;
+          }
+          rs_arrive_scal(RC ? 96 : 64);
+        } else {
+          for (int t = threadIdx.x; t < nr; t += 32 * (nrow_w - 1)) {
+            VT tv = vj[t], u = sw[t];
+#pragma unroll 4
+            for (int i = 0; i < nb; ++i) {
+              const VT v = qv(q, i)[t];
+              tv -= rs_head(S3[i]) * v;
+              u -= rs_head(s1[i]) * v;
+            }
+            vn[t] = tv;
+            sw[t] = u;
+          }
+        }
+        rs_bar_rows(32 * nrow_w);
+        const bool lost = s_lost == 2, brk = s_lost != 0;
+        if (!lost) {
+          const VT inu = s_inu, ib = s_ib, vh = s_vh;
+          for (int t = threadIdx.x; t < nr; t += 32 * nrow_w) {
+            const VT tv = vn[t], u = sw[t];
+            const VT vt = tv * inu;
+            vj[t] = vt;
+            const VT zz = brk ? (VT)0 : (u - vh * vt) * ib;
+            vn[t] = zz;
+            Z[(size_t)(j + 1) * zst + t] = zz;
+            zb[c0r + t] = zz * swt[t];
+          }
+          rs_bar_rows(32 * nrow_w);
+          // a' = Q_i^T z_{j+1} (i <= nb, v_j included), |z_{j+1}|^2, obstacle sums
+          float4* p3 = part3((j + 1) & 1);
+          const int nrow = nb + 2 + nobs;
+          for (int i = warp; i < nrow; i += nrow_w) {
+            if (i <= nb + 1) {
+              const VT* qi = qv(q, i);
+              typename AZ::T s = AZ::zero();
+              for (int t = lane; t < nr; t += 32) s = AZ::mad(s, qi[t], vn[t]);
+              s = AZ::warp(s);
+              if (lane == 0) rs_put(p3, (size_t)i * G + blockIdx.x, AZ::split(s));
+            } else {
+              const int o = i - (nb + 2);
+              const int a0 = max(0, a.obs_off[o] - c0r), a1 = min(nr, a.obs_off[o + 1] - c0r);
+              typename AC::T s = AC::zero();
+              for (int t = a0 + lane; t < a1; t += 32) s = AC::addv(s, vn[t]);
+              s = AC::warp(s);
+              if (lane == 0) rs_put(p3, (size_t)i * G + blockIdx.x, AC::split(s));
+            }
+          }
         }
       }
       if (!rs_barrier(a, epoch, &s_ok)) { leave(); return; }
-      if (now && s_done) {
+      if ((!a.lag || s_lost != 0 || j + 1 >= m) && s_done) {   // the test was made in this phase
         k = s_iters;
         break;
       }
@@ -1042,35 +1256,29 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
     if (k > 0) {
       PS* pa = s3 + (size_t)(k & 1) * s3n;                    // dots of z_k, q + k + 1
       {
-        PX ld3[AC::LD];
-        rs_load<VT>(part3[k & 1], q + k + 1, G, ld3);
-        rs_reduce<VT>(part3[k & 1], q + k + 1, G, ld3, pa, blockDim.x);
+        typename AZ::X ld3[AZ::LD];
+        rs_load<AZ, 16>(part3(k & 1), q + k + 1, G, ld3);
+        rs_reduce<AZ, 16>(part3(k & 1), q + k + 1, G, ld3, pa, blockDim.x);
       }
       __syncthreads();
-      auto pv = [&](int i) -> double { return AC::value(AC::unpack(pa[i])); };
+      auto pv = [&](int i) -> double { return rs_value(pa[i]); };
       double* hl = h_fin;                                     // column k - 1
       double* bl = h_braw;                                    // becomes its C-part
       auto Rent = [&](int i, int c) -> double { return c == k - 1 ? hl[i] : Hm[(size_t)c * (c + 1) / 2 + i]; };
       auto Bent = [&](int l, int i) -> double { return i == k - 1 ? bl[l] : Bm[(size_t)i * RS_RQ + l]; };
       if (warp == 0) {
-        PT ta = AC::zero();
-        for (int i = lane; i < q + k; i += 32) ta = ta + AC::unpack(pa[i]) * AC::unpack(pa[i]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ta = ta + AC::shfl(ta, o);
-        const PT nu2 = AC::unpack(pa[q + k]) - ta;
-        const PT inu = AC::rsqrt_pos(nu2);
-        const double nu = AC::value(nu2 * inu);
         const double bk = h_raw[k];
         for (int i = lane; i < k; i += 32) hl[i] = fma(bk, pv(q + i), h_raw[i]);
         for (int l = lane; l < q; l += 32) bl[l] = fma(bk, pv(l), bl[l]);
         __syncwarp();
         const double u = givens_apply_warp(hl, h_cs, h_sn, k - 1);
+        rs_bar_scal(64);
+        const double nu = s_nu;
         double c, s, rr, ir;
         rs_givens(u, bk * nu, c, s, rr, ir);
         if (lane == 0) {
           hl[k - 1] = rr;
           h_rinv[k - 1] = ir;
-          s_inu = AC::head(inu);
           s_c = (VT)c;
           s_s = (VT)s;
         }
@@ -1111,6 +1319,16 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
           tq[l] = t;
           f1[m + 2 + l] = (VT)t;
         }
+      } else if (warp == 2) {   // the norm of z_k less its parts, beside warp 0's rotations
+        double ta = 0.0;
+        for (int i = lane; i < q + k; i += 32) ta = fma(pv(i), pv(i), ta);
+        ta = warp_sum(ta);
+        const double nu2 = pv(q + k) - ta, inu = rs_rsqrt_pos(nu2);
+        if (lane == 0) {
+          s_nu = nu2 * inu;
+          s_inu = (VT)inu;
+        }
+        rs_arrive_scal(64);
       } else if (warp == 1 && ext) {
         asm volatile("bar.sync 2, 64;" ::: "memory");
         if (lane < k) {
@@ -1185,7 +1403,7 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
             const PS* pa = s3 + (size_t)(k & 1) * s3n;
             VT vk = V[(size_t)k * R + t];
 #pragma unroll 4
-            for (int l = 0; l < q + k; ++l) vk -= AC::head(AC::unpack(pa[l])) * qv(q, l)[t];
+            for (int l = 0; l < q + k; ++l) vk -= rs_head(pa[l]) * qv(q, l)[t];
             vk *= s_inu;
             VT cur = V[t];
             for (int i = 0; i < k; ++i) {
@@ -1283,14 +1501,17 @@ static bool rs_plan(const bie_ctx* c, const bie_solve_opts* o, int nobs, RsPlan&
   L.red = take(4 * (4 * 32 + R + 4));
   L.xo = take(8 * 2 * R);
   L.wt = take(vt * 3 * R);
-  L.s1 = take(8 * (m + 2 + RS_RQ));
-  L.s3 = take(8 * 2 * (m + 2 + RS_RQ + (size_t)nobs));
+  const size_t ps = f64 ? sizeof(RsAcc<double, true>::S) : sizeof(RsAcc<float, true>::S);
+  L.s1 = take(ps * (m + 2 + RS_RQ));
+  L.s3 = take(ps * 2 * (m + 2 + RS_RQ + (size_t)nobs));
   L.cs = take(8 * m);
   L.sn = take(8 * m);
   L.g = take(8 * (m + 1));
   L.hraw = take(8 * (m + 2));
   L.braw = take(8 * RS_RQ);
   L.hfin = take(8 * (m + 2));
+  L.hnew = take(8 * (m + 2));
+  L.bnew = take(8 * RS_RQ);
   L.rinv = take(8 * (m + 1));
   L.H = take(8 * (size_t)m * (m + 1) / 2);
   L.B = take(8 * rq * m);
@@ -1412,13 +1633,14 @@ bie_status resident_launch(bie_ctx* c, const bie_solve_opts* o, double* x, const
   // one exchange buffer: z_j, xh, xl (zero past N), partial sums, barrier
   const size_t ldb = 8 * (size_t)c->ld;
   a.prow = a.m + 2 + RS_RQ + a.nobs;
-  const size_t pbytes = (ir ? 8 : 16) * (size_t)a.prow * P.G;
+  const size_t pbytes = 3 * sizeof(float4) * (size_t)a.prow * P.G;
   unsigned char* xb;
   unsigned* bar;
   BIE_GET(c, unsigned char, "rs_x", 3 * ldb, xb);
-  BIE_GET(c, unsigned char, "rs_part", 3 * pbytes + 8 * (size_t)P.G, a.part1);
-  a.part3 = (unsigned char*)a.part1 + pbytes;
-  a.partn = (double*)((unsigned char*)a.part1 + 3 * pbytes);
+  unsigned char* pb;
+  BIE_GET(c, unsigned char, "rs_part", pbytes + 8 * (size_t)P.G, pb);
+  a.part = (float4*)pb;
+  a.partn = (double*)(pb + pbytes);
   BIE_GET(c, unsigned, "rs_bar", 4, bar);
   if (c->rs_bar != bar) {
     BIE_CUDA_TRY(c, cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), c->stream));
