@@ -310,3 +310,31 @@ def test_matmat_full_full_size(P):
         assert np.all(np.abs(Yd.cpu().numpy()[:, rows] - ref) <= 1e-13 * scale)
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("n,nrhs", [(1501, 5), (2944, 12), (1501, 20)])
+def test_repeated_solves_give_the_same_bits(P, n, nrhs):
+    """Columns whose cycles end at different steps (smooth and rough data of several sizes):
+    every run takes the same steps and gives the same bits."""
+    import torch
+    g, f, _ = W.random_geometry(np.random.default_rng(n), n)
+    rng = np.random.default_rng(nrhs)
+    PH = np.stack([W.filtered_noise(rng, g.M[0], 10.0 ** rng.uniform(-4, 1), int(rng.integers(1, 60)))
+                   for _ in range(nrhs)])
+    PH[1] = 0.3                                       # a constant: few steps
+    prob = P.Problem(g, f, PH[0])
+    try:
+        prob.assemble("fp16_ir")
+        ph = torch.as_tensor(PH, device="cuda").contiguous()
+        om = torch.empty((nrhs, g.N), dtype=torch.float64, device="cuda")
+        U = torch.empty((nrhs, g.M[0]), dtype=torch.float64, device="cuda")
+        first = None
+        for _ in range(12):
+            infos = P.bie_solve_multi(prob.ctx, ph, om, U)
+            steps = [i.iters for i in infos]
+            if first is None:
+                first = (om.clone(), U.clone(), steps)
+                assert len(set(steps)) > 1
+            assert steps == first[2] and torch.equal(om, first[0]) and torch.equal(U, first[1])
+    finally:
+        prob.close()

@@ -201,3 +201,66 @@ def test_failed_solve_leaves_U_and_psi_alone(P, prec):
         assert P.bie_solve(prob.ctx, prob.phit, om, U, psi).converged
     finally:
         prob.close()
+
+
+def _both_solvers(P, prob, b, N, **kw):
+    """(status, x, info) of the one-kernel solver and of the kernel-by-kernel one."""
+    import torch
+    out = []
+    for prof in (0, 1):
+        P.bie_set_profiling(prob.ctx, prof)
+        om = torch.full((N,), np.nan, dtype=torch.float64, device="cuda")
+        try:
+            info, st = P.bie_solve_b(prob.ctx, b, om, P.bie_default_opts(**kw)), 0
+        except P.BieError as e:
+            info, st = None, e.status
+        out.append((st, om, info))
+    P.bie_set_profiling(prob.ctx, 0)
+    return out
+
+
+@pytest.mark.parametrize("n,prec", [(6655, "fp16_ir"), (6703, "fp16_ir"), (6703, "bf16_ir"), (4740, "fp32_ir"),
+                                    (4801, "fp32_ir")])
+def test_one_kernel_solve_around_the_l2_size(P, n, prec):
+    """Just below and just above 90 MB of inner storage, where a row takes one warp and
+    the heads of the rows leave shared memory; ragged sizes."""
+    import torch
+    g, f, ph = W.random_geometry(np.random.default_rng(n), n)
+    assert g.N % 64 != 0
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        b = torch.empty(g.N, dtype=torch.float64, device="cuda")
+        P.bie_rhs(prob.ctx, prob.phit, b)
+        (s0, x0, i0), (s1, x1, i1) = _both_solvers(P, prob, b, g.N)
+        assert s0 == s1 == 0 and i0.converged and i1.converged
+        assert float((x0 - x1).norm() / x1.norm()) <= 1e-12
+    finally:
+        prob.close()
+
+
+@pytest.mark.parametrize("M0,M1,Mo", [(20, 12, []), (41, 29, [23, 25]), (640, 330, [161, 170])])
+@pytest.mark.parametrize("prec", ["fp64", "fp32_ir", "bf16_ir"])
+def test_option_sets_that_must_converge_and_that_must_not(P, M0, M1, Mo, prec):
+    """The option sets of the comparison that have to converge do, and where both solvers run
+    out of cycles their iterates are equally good: residuals within a factor of 2."""
+    import torch
+    g, f, ph = _geometry(M0, M1, Mo)
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        b = torch.empty(g.N, dtype=torch.float64, device="cuda")
+        P.bie_rhs(prob.ctx, prob.phit, b)
+        for kw in ({}, {"row_flip": 0}, {"restart": 200}, {"rtol": 1e-10, "inner_tol": 1e-2}):
+            for st, _, info in _both_solvers(P, prob, b, g.N, **kw):
+                assert st == 0 and info.converged, kw
+        y = torch.empty_like(b)
+        for kw in ({"restart": 3, "max_cycles": 2}, {"restart": 2, "max_cycles": 3}, {"restart": 5, "max_cycles": 1}):
+            res = []
+            for st, x, _ in _both_solvers(P, prob, b, g.N, **kw):
+                assert st == P.BIE_ERR_NOCONV, kw
+                P.bie_matvec(prob.ctx, 1, x, y)
+                res.append(float((b - y).norm() / b.norm()))
+            assert 1e-13 < max(res) < 1.0 and max(res) <= 2.0 * min(res), (kw, res)
+    finally:
+        prob.close()
