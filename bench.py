@@ -390,6 +390,9 @@ def _config(args, g):
 # ---------------------------------------------------------------------------
 # GPU arm
 # ---------------------------------------------------------------------------
+# the solver of row-partitioned contexts, of more than 16384 unknowns and under profiling
+STEPWISE = "kernel_by_kernel"
+
 
 def run_ours(args):
     import numpy as np
@@ -432,6 +435,7 @@ def run_ours(args):
         torch.cuda.synchronize(dev)
         if profile:
             P.bie_set_profiling(ctx, True)
+        n0 = P.bie_get_profile(ctx).as_dict()["kernel_launches"]
         barrier(ws)
         torch.cuda.synchronize(dev)
         e0 = torch.cuda.Event(enable_timing=True)
@@ -446,11 +450,12 @@ def run_ours(args):
             torch.cuda.synchronize(dev)
         barrier(ws)
         ms = e0.elapsed_time(e1)
-        prof = P.bie_get_profile(ctx).as_dict() if profile else None
+        prof = P.bie_get_profile(ctx).as_dict()
+        launches = prof["kernel_launches"] - n0   # of the library, inside the timed region
         if profile:
             P.bie_set_profiling(ctx, False)
         ms = max_over_ranks(ms, ws, dev)
-        return ms, infos, prof
+        return ms, infos, prof if profile else None, launches
 
     # --- every storage scheme, briefly, for the variant table
     variants = {}
@@ -458,16 +463,18 @@ def run_ours(args):
         K = max(2, min(args.steps, 5)) if prec != args.precision else 0
         if K == 0:
             continue
-        ms, infos, vprof = timed(prec, K, 1, profile=(prec == "fp64"))
+        ms, infos, _, _ = timed(prec, K, 1)
         variants[prec] = _variant_entry(ms, K, infos, ws)
         variants[prec]["U_checksum"] = float(U.double().sum().item())
         if prec == "fp64":
-            # FP64 storage: 2 N^2 flops per product against the FP64 pipe: the
-            # DFMA rate measured on this machine's GB300 (independent FMA chains at
-            # full occupancy) and the nominal 1.25 TFLOP/s
+            # the kernel-by-kernel solver's product (profiling selects that solver; the
+            # time above is the one-kernel solver's).  FP64 storage: 2 N^2 flops per
+            # product against the FP64 pipe: the DFMA rate measured on the GB300
+            # (independent FMA chains at full occupancy) and the nominal 1.25 TFLOP/s
+            vprof = timed(prec, 2, 1, profile=True)[2]
             gms = vprof["ms_gemv_inner"] / max(1, vprof["n_gemv_inner"])
             fl = 2.0 * N * N / (gms * 1e-3)
-            variants[prec]["gemv_f64"] = {"avg_ms": gms, "launches": vprof["n_gemv_inner"],
+            variants[prec]["gemv_f64"] = {"solver": STEPWISE, "avg_ms": gms, "launches": vprof["n_gemv_inner"],
                                           "TFLOPs": fl / 1e12,
                                           "peak_TFLOPs_measured": FP64_FMA_TFLOPS,
                                           "frac_of_measured": fl / (FP64_FMA_TFLOPS * 1e12),
@@ -478,15 +485,23 @@ def run_ours(args):
     # --- the headline: the chosen scheme, K timed steps with nothing but the work
     hb_peak, peak_kind = _peaks()
     sampler = ClockSampler(local) if rank == 0 else None
-    ms, infos, _ = timed(args.precision, args.steps, args.warmup, profile=False, clocks=sampler)
+    ms, infos, _, launches = timed(args.precision, args.steps, args.warmup, clocks=sampler)
     variants[args.precision] = _variant_entry(ms, args.steps, infos, ws)
     value = job_throughput(args.steps, ws, ms / 1e3)
-    # --- the same K steps again with CUDA events around every hot launch on the
-    # library's stream (kernel shares, roofline, launch count); the events add
-    # ~2% to a step, so the headline pass above runs without them
-    ms_prof, _, prof = timed(args.precision, args.steps, 1, profile=True)
     om_head = omega.cpu().numpy().copy()
     U_head = U.cpu().numpy().copy()
+    # --- the solver alone as the steps above run it, on the last step's system
+    bvec = torch.empty(N, dtype=torch.float64, device=dev)
+    P.bie_rhs(ctx, phit, bvec)
+    xvec = torch.empty_like(bvec)
+    n0 = P.bie_get_profile(ctx).as_dict()["kernel_launches"]
+    solve_ms, solve_info = _events_ms(stream, lambda: P.bie_solve_b(ctx, bvec, xvec, opts), args.steps,
+                                      warm=3)
+    solve_launches = (P.bie_get_profile(ctx).as_dict()["kernel_launches"] - n0) / (args.steps + 3)
+    # --- the same K steps once more with CUDA events around every hot launch on the
+    # library's stream.  Profiling selects the kernel-by-kernel solver, so what this pass
+    # says about products is of that solver (7% slower per step here, events included)
+    ms_prof, infos_prof, prof, _ = timed(args.precision, args.steps, 1, profile=True)
 
     # agreement between the headline scheme and the plain FP64 scheme
     diff = None
@@ -537,7 +552,9 @@ def run_ours(args):
     if rank != 0:
         return 0
 
-    # --- roofline of the dominant kernel (by accumulated time)
+    # --- roofline of the dominant kernel: the solver, its matrix products' bytes (the
+    # profiled pass counts them; both solvers take the same steps and residuals) over its
+    # whole duration
     kinds = {
         "gemv_inner": (prof["ms_gemv_inner"], prof["n_gemv_inner"], prof["bytes_gemv_inner"]),
         "gemv_full": (prof["ms_gemv_full"], prof["n_gemv_full"], prof["bytes_gemv_full"]),
@@ -547,26 +564,40 @@ def run_ours(args):
     }
     step_ms = ms_prof / args.steps
     shares = {k: (v[0] / args.steps) / step_ms for k, v in kinds.items()}
-    gemv_key = {"fp32_ir": "k_gemv_lowp<float>", "fp16_ir": "k_gemv_lowp<__half>",
-                "bf16_ir": "k_gemv_lowp<__nv_bfloat16>", "fp64": "k_gemv_f64"}[args.precision]
+    tname = {"fp32_ir": "float", "fp16_ir": "__half", "bf16_ir": "__nv_bfloat16", "fp64": "double"}[args.precision]
+    one_kernel = solve_launches == 1.0
+    solve_bytes = sum(n * b for _, n, b in (kinds["gemv_inner"], kinds["gemv_full"], kinds["gemv_hi"])) / args.steps
+    achieved_solve = solve_bytes / (solve_ms * 1e-3) / 1e9
+    roofline = {"bound": "hbm",
+                "kernel": f"k_resident<{tname}>" if one_kernel else STEPWISE,
+                "achieved": achieved_solve, "peak": hb_peak, "peak_kind": peak_kind, "unit": "GB/s",
+                "frac": achieved_solve / hb_peak, "traffic": None,
+                "avg_launch_ms": solve_ms, "launches": args.steps if one_kernel else None,
+                "algorithmic_bytes_per_launch": solve_bytes,
+                "iters": solve_info.iters, "same_steps_as_counted": solve_info.iters == infos_prof[-1].iters,
+                "timed_pass": "bie_solve_b on the headline system, events around K calls, no profiling: all "
+                              "products of a solve over its whole duration, its Gram-Schmidt work, barriers "
+                              "and the host's wait included"}
+    # one product of the kernel-by-kernel solver (row-partitioned contexts, more than 16384 unknowns)
+    gemv_key = "k_gemv_f64" if args.precision == "fp64" else f"k_gemv_lowp<{tname}>"
     avg_ms = prof["ms_gemv_inner"] / max(1, prof["n_gemv_inner"])
     achieved = prof["bytes_gemv_inner"] / (avg_ms * 1e-3) / 1e9
     full_avg = prof["ms_gemv_full"] / max(1, prof["n_gemv_full"])
-    roofline = {"bound": "hbm", "kernel": gemv_key, "achieved": achieved, "peak": hb_peak,
-                "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / hb_peak,
-                "traffic": _traffic(gemv_key), "avg_launch_ms": avg_ms,
-                "launches": prof["n_gemv_inner"],
-                "algorithmic_bytes_per_launch": prof["bytes_gemv_inner"],
-                "timed_pass": "the K headline steps repeated with an event pair around each launch"}
+    roofline_product = {"bound": "hbm", "solver": STEPWISE, "kernel": gemv_key, "achieved": achieved,
+                        "peak": hb_peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / hb_peak,
+                        "traffic": _traffic(gemv_key), "avg_launch_ms": avg_ms,
+                        "launches": prof["n_gemv_inner"],
+                        "algorithmic_bytes_per_launch": prof["bytes_gemv_inner"],
+                        "timed_pass": "the K headline steps repeated with an event pair around each launch"}
     if args.precision != "fp64":
         # the library's Gram-Schmidt kernels fetch the first quarter-L2 of the
         # stored matrix into L2 while HBM is otherwise idle; that part of each
         # launch's stream comes from L2, the rest from HBM
         l2 = int(getattr(torch.cuda.get_device_properties(0), "L2_cache_size", 0))
         pf = min(l2 // 4, int(prof["bytes_gemv_inner"])) // 16 * 16
-        roofline["l2_prefetched_bytes_per_launch"] = pf
-        roofline["frac_hbm_part"] = ((prof["bytes_gemv_inner"] - pf) / (avg_ms * 1e-3) / 1e9
-                                     / hb_peak)
+        roofline_product["l2_prefetched_bytes_per_launch"] = pf
+        roofline_product["frac_hbm_part"] = ((prof["bytes_gemv_inner"] - pf) / (avg_ms * 1e-3) / 1e9
+                                             / hb_peak)
     asm_avg_ms = prof["ms_assemble"] / max(1, prof["n_assemble"])
     asm_inst = _counters("k_assemble_pairs<dfl>", "warp_instructions_per_launch")
     asm_peak = ISSUE_SLOTS_PER_CYCLE * _peak_clock_mhz() * 1e6
@@ -588,6 +619,13 @@ def run_ours(args):
                     # the stores alone (A hi/lo/16 + surface U-matrix hi/lo) at the HBM peak
                     "hbm_write_ms_at_peak": (N * N * 10.0 + M0 * N * 8.0) / (hb_peak * 1e9) * 1e3}
     kernels = {
+        # of the headline steps: the solver alone, and the kernels both solvers share
+        "headline": {"ms_per_step": ms / args.steps, "solver_ms": solve_ms,
+                     "solver_share": solve_ms / (ms / args.steps),
+                     "assemble_ms": kinds["assemble"][0] / args.steps,
+                     "velocity_ms": kinds["velocity"][0] / args.steps},
+        # of the profiled steps
+        "solver": STEPWISE,
         "gemv_inner": {"ms_per_step": kinds["gemv_inner"][0] / args.steps, "share": shares["gemv_inner"],
                        "launches_per_step": prof["n_gemv_inner"] / args.steps, "avg_ms": avg_ms,
                        "GBps": achieved},
@@ -626,6 +664,7 @@ def run_ours(args):
         "data": "synthetic",
         "config": _config(args, g),
         "roofline": roofline,
+        "roofline_stepwise_product": roofline_product,
         "roofline_assembly": roofline_asm,
         "kernels": kernels,
         "variants": variants,
@@ -633,7 +672,7 @@ def run_ours(args):
                      "iters": infos[-1].iters, "cycles": infos[-1].cycles},
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": int(prof["kernel_launches"]),
+        "gpu_launches": int(launches),
         "clocks": clocks,
         "rows": rows,
     }
