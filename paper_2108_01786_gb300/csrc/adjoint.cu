@@ -555,14 +555,11 @@ static bie_status spectral_d(bie_ctx* c, const double2* x, const double2* tw, do
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  int s = 0;
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J1.j[J1.n++] = DftJob{M, M1, M / M1, o, o, o, 3, s};
-    J2.j[J2.n++] = DftJob{M, M1, M / M1, o, o, o, 1, s};
-    s += M;
+    J1.j[J1.n++] = DftJob{M, M1, o, o, o, 3};
+    J2.j[J2.n++] = DftJob{M, M1, o, o, o, 1};
   }
-  J1.total = J2.total = s;
   bie_status st = dft_run(c, J1, nullptr, x, Y, X1);
   if (st != BIE_OK) return st;
   return dft_run(c, J2, nullptr, X1, Y, X2);
@@ -696,23 +693,18 @@ extern "C" bie_status bie_backward(bie_ctx* c, const double* omega, const double
     DftJobs J1, J2;
     memset(&J1, 0, sizeof(J1));
     memset(&J2, 0, sizeof(J2));
-    int t = 0;
     for (int k = 0; k < c->nb; ++k) {
       const int M = c->M[k], M1 = c->fft_m1[k], o0 = c->off[k];
-      J1.j[J1.n++] = DftJob{M, M1, M / M1, o0, o0, o0, 0, t};
-      J2.j[J2.n++] = DftJob{M, M1, M / M1, o0, o0, o0, 1, t};
-      t += M;
+      J1.j[J1.n++] = DftJob{M, M1, o0, o0, o0, 0};
+      J2.j[J2.n++] = DftJob{M, M1, o0, o0, o0, 1};
     }
-    J1.j[J1.n++] = DftJob{M0, c->fft_m1[0], M0 / c->fft_m1[0], N, N, 0, 0, t};
-    J2.j[J2.n++] = DftJob{M0, c->fft_m1[0], M0 / c->fft_m1[0], N, N, 0, 2, t};
-    t += M0;
+    J1.j[J1.n++] = DftJob{M0, c->fft_m1[0], N, N, 0, 0};
+    J2.j[J2.n++] = DftJob{M0, c->fft_m1[0], N, N, 0, 2};
     for (int k = 0; k < c->nb; ++k) {
       const int M = c->M[k], M1 = c->fft_m1[k], o0 = c->off[k];
-      J1.j[J1.n++] = DftJob{M, M1, M / M1, N + M0 + o0, N + M0 + o0, o0, 0, t};
-      J2.j[J2.n++] = DftJob{M, M1, M / M1, N + M0 + o0, N + M0 + o0, o0, 1, t};
-      t += M;
+      J1.j[J1.n++] = DftJob{M, M1, N + M0 + o0, N + M0 + o0, o0, 0};
+      J2.j[J2.n++] = DftJob{M, M1, N + M0 + o0, N + M0 + o0, o0, 1};
     }
-    J1.total = J2.total = t;
     s = dft_run(c, J1, xin, nullptr, dY, dX1);
     if (s != BIE_OK) return s;
     s = dft_run(c, J2, nullptr, dX1, dY, dX2);

@@ -406,7 +406,7 @@ bie_status dft_tables(bie_ctx* c) {
     if (q == 0) continue;
     k_bl_tables<<<(q + 63) / 64, 64, 0, c->stream>>>(c->M[k], q, chirp + c->off[k], F + o, twq + o);
     BIE_LAUNCH_CHECK(c, "k_bl_tables");
-    J.j[J.n++] = DftJob{q, largest_divisor(q), q / largest_divisor(q), o, o, o, 3, 0};
+    J.j[J.n++] = DftJob{q, largest_divisor(q), o, o, o, 3};
   }
   const cudaError_t e = dft_run_plain(c->stream, J, nullptr, F, twq, Y, bhat);
   if (e != cudaSuccess) return ctx_cuda(c, e, "k_dft (tables)");

@@ -3,7 +3,7 @@
 #include "common.cuh"
 
 struct DftJob {
-  int M, M1, M2;
+  int M, M1;
   int off_in;    // input offset (real omega for mode 0, spectrum for modes 1/2)
   int off_out;   // output offset in the complex work array
   int off_tw;    // offset of the boundary's nodes (its tables: e^{-2 pi i j / M}, j < M)
@@ -12,11 +12,9 @@ struct DftJob {
                  // (second derivative); 6: conj(rho(k) X) (filter of eq. filter);
                  // 7: conj(X/(ik)), zero at k = 0 (zero-mean antiderivative);
                  // 8: real input from the second input array
-  int start;     // first global element of this job
 };
 struct DftJobs {
   int n;
-  int total;
   DftJob j[2 * BIE_MAXB + 2];
 };
 

@@ -3,7 +3,7 @@
 // the conserved energy of eq. E:formula (Sec. 5.2).
 //
 // One right-hand-side evaluation: the surface zeta_0 = alpha + i eta with
-// zeta_0' and zeta_0'' from spectral derivatives of eta (FP64 four-step DFT),
+// zeta_0' and zeta_0'' from spectral derivatives of eta (FP64 transforms, dft.cu),
 // the node tables rebuilt, the matrix assembled and the system solved by the
 // library's own kernels, then eta_t = s_alpha U and phi~_t of eq. phitileq
 // (V = eta_alpha U, C(t) = 0, rho = 1) in one FP64 pass over the surface.
@@ -52,22 +52,18 @@ __device__ __forceinline__ dfl df_shfl_sum(dfl v) {
 
 // y = [eta | phi~] (2 M_0) -> X2 = [eta_alpha | phi~_alpha | eta_alpha_alpha] x M_0
 bie_status graph_derivs(bie_ctx* c, const double* y, double2* X2) {
-  const int M0 = c->M[0], M1 = c->fft_m1[0], M2 = M0 / M1;
+  const int M0 = c->M[0], M1 = c->fft_m1[0];
   double2 *dY, *dX1;
   BIE_GET(c, double2, "ev_Y", 3 * (size_t)M0, dY);
   BIE_GET(c, double2, "ev_X1", 2 * (size_t)M0, dX1);
-  bool oom = false;
-  if (oom) return ctx_fail(c, BIE_ERR_OOM, "evolve: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  J1.j[J1.n++] = DftJob{M0, M1, M2, 0, 0, 0, 0, 0};
-  J1.j[J1.n++] = DftJob{M0, M1, M2, M0, M0, 0, 0, M0};
-  J1.total = 2 * M0;
-  J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 0, 0, 1, 0};
-  J2.j[J2.n++] = DftJob{M0, M1, M2, M0, M0, 0, 1, M0};
-  J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 2 * M0, 0, 5, 2 * M0};
-  J2.total = 3 * M0;
+  J1.j[J1.n++] = DftJob{M0, M1, 0, 0, 0, 0};
+  J1.j[J1.n++] = DftJob{M0, M1, M0, M0, 0, 0};
+  J2.j[J2.n++] = DftJob{M0, M1, 0, 0, 0, 1};
+  J2.j[J2.n++] = DftJob{M0, M1, M0, M0, 0, 1};
+  J2.j[J2.n++] = DftJob{M0, M1, 0, 2 * M0, 0, 5};
   if (bie_status sd = dft_run(c, J1, y, nullptr, dY, dX1)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, X2)) return sd;
   return BIE_OK;
@@ -394,7 +390,7 @@ bie_status pot_run(bie_ctx* c, bool all, const FlowParams& F, const PairNodes& n
 bie_status energy_run(bie_ctx* c, const double* phit, const double* omega, double tau, double g,
                       double* E_dev) {
   BIE_NVTX("energy");
-  const int N = c->N, M0 = c->M[0], M1 = c->fft_m1[0], M2 = M0 / M1;
+  const int N = c->N, M0 = c->M[0], M1 = c->fft_m1[0];
   double2 *dY, *dX1, *dX2;
   double *psi0, *psik;
   BIE_GET(c, double2, "en_Y", 2 * (size_t)M0, dY);
@@ -419,11 +415,10 @@ bie_status energy_run(bie_ctx* c, const double* phit, const double* omega, doubl
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  J1.j[J1.n++] = DftJob{M0, M1, M2, 0, 0, 0, 0, 0};
-  J1.j[J1.n++] = DftJob{M0, M1, M2, 0, M0, 0, 8, M0};
-  J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 0, 0, 4, 0};
-  J2.j[J2.n++] = DftJob{M0, M1, M2, M0, M0, 0, 1, M0};
-  J1.total = J2.total = 2 * M0;
+  J1.j[J1.n++] = DftJob{M0, M1, 0, 0, 0, 0};
+  J1.j[J1.n++] = DftJob{M0, M1, 0, M0, 0, 8};
+  J2.j[J2.n++] = DftJob{M0, M1, 0, 0, 0, 4};
+  J2.j[J2.n++] = DftJob{M0, M1, M0, M0, 0, 1};
   if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX1, 1, 0, 0, phit)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   const Blocks B = make_blocks(c);
@@ -461,20 +456,17 @@ __global__ void k_take_real_mode(int n, int M0, const double2* __restrict__ X, d
 
 // eq. filter on nv consecutive surface vectors of x (in place)
 bie_status filter_run(bie_ctx* c, double* x, int nv) {
-  const int M0 = c->M[0], M1 = c->fft_m1[0], M2 = M0 / M1;
+  const int M0 = c->M[0], M1 = c->fft_m1[0];
   double2 *dY, *dX1;
   BIE_GET(c, double2, "fl_Y", 2 * (size_t)M0, dY);
   BIE_GET(c, double2, "fl_X1", 2 * (size_t)M0, dX1);
-  bool oom = false;
-  if (oom) return ctx_fail(c, BIE_ERR_OOM, "filter: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
   for (int v = 0; v < nv; ++v) {
-    J1.j[J1.n++] = DftJob{M0, M1, M2, v * M0, v * M0, 0, 0, v * M0};
-    J2.j[J2.n++] = DftJob{M0, M1, M2, v * M0, v * M0, 0, 6, v * M0};
+    J1.j[J1.n++] = DftJob{M0, M1, v * M0, v * M0, 0, 0};
+    J2.j[J2.n++] = DftJob{M0, M1, v * M0, v * M0, 0, 6};
   }
-  J1.total = J2.total = nv * M0;
   const unsigned gb = (unsigned)((nv * M0 + 255) / 256);
   if (bie_status sd = dft_run(c, J1, x, nullptr, dY, dX1)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX1)) return sd;
@@ -486,20 +478,17 @@ bie_status filter_run(bie_ctx* c, double* x, int nv) {
 // forward (mode 0) then inverse passes with modes m0, m1 on two stacked
 // surface vectors x = [a | b]: out = [D_m0 a | D_m1 b] (real part / M_0 taken by the caller)
 bie_status dft_pair(bie_ctx* c, const double* x, int m0, int m1, double2* out) {
-  const int M0 = c->M[0], M1 = c->fft_m1[0], M2 = M0 / M1;
+  const int M0 = c->M[0], M1 = c->fft_m1[0];
   double2 *dY, *dX1;
   BIE_GET(c, double2, "hp_Y", 2 * (size_t)M0, dY);
   BIE_GET(c, double2, "hp_X1", 2 * (size_t)M0, dX1);
-  bool oom = false;
-  if (oom) return ctx_fail(c, BIE_ERR_OOM, "dft: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  J1.j[J1.n++] = DftJob{M0, M1, M2, 0, 0, 0, 0, 0};
-  J1.j[J1.n++] = DftJob{M0, M1, M2, M0, M0, 0, 0, M0};
-  J2.j[J2.n++] = DftJob{M0, M1, M2, 0, 0, 0, m0, 0};
-  J2.j[J2.n++] = DftJob{M0, M1, M2, M0, M0, 0, m1, M0};
-  J1.total = J2.total = 2 * M0;
+  J1.j[J1.n++] = DftJob{M0, M1, 0, 0, 0, 0};
+  J1.j[J1.n++] = DftJob{M0, M1, M0, M0, 0, 0};
+  J2.j[J2.n++] = DftJob{M0, M1, 0, 0, 0, m0};
+  J2.j[J2.n++] = DftJob{M0, M1, M0, M0, 0, m1};
   if (bie_status sd = dft_run(c, J1, x, nullptr, dY, dX1)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, out)) return sd;
   return BIE_OK;
@@ -731,17 +720,14 @@ bie_status dft_blocks(bie_ctx* c, const double* x, int mode, double2* out) {
   double2 *dY, *dX1;
   BIE_GET(c, double2, "db_Y", N, dY);
   BIE_GET(c, double2, "db_X1", N, dX1);
-  bool oom = false;
-  if (oom) return ctx_fail(c, BIE_ERR_OOM, "dft: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J1.j[J1.n++] = DftJob{M, M1, M / M1, o, o, o, 0, o};
-    J2.j[J2.n++] = DftJob{M, M1, M / M1, o, o, o, mode, o};
+    J1.j[J1.n++] = DftJob{M, M1, o, o, o, 0};
+    J2.j[J2.n++] = DftJob{M, M1, o, o, o, mode};
   }
-  J1.total = J2.total = N;
   if (bie_status sd = dft_run(c, J1, x, nullptr, dY, dX1)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, out)) return sd;
   return BIE_OK;

@@ -511,24 +511,18 @@ static bie_status boundary_values(bie_ctx* c, const double* omega, double2** f64
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  int s1 = 0, s2 = 0;
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J1.j[J1.n++] = DftJob{M, M1, M / M1, o, o, o, 0, s1};
-    s1 += M;
+    J1.j[J1.n++] = DftJob{M, M1, o, o, o, 0};
   }
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J2.j[J2.n++] = DftJob{M, M1, M / M1, o, o, o, 1, s2};
-    s2 += M;
+    J2.j[J2.n++] = DftJob{M, M1, o, o, o, 1};
   }
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J2.j[J2.n++] = DftJob{M, M1, M / M1, o, N + o, o, 2, s2};
-    s2 += M;
+    J2.j[J2.n++] = DftJob{M, M1, o, N + o, o, 2};
   }
-  J1.total = s1;
-  J2.total = s2;
   if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX1)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   k_gamma_extract<<<(N + 255) / 256, 256, 0, c->stream>>>(B, dX2, gc, hg, cf);

@@ -267,7 +267,7 @@ bie_status vgemv_run(bie_ctx* c, const float* xh, const float* xl, const double*
                      double** ypart_out, int* npanel_out);
 
 // omega'/M_k as double-float hi/lo arrays (zero padded to ld) and H omega_0',
-// by the FP64 four-step DFT: the inputs of the U-matrix product
+// by FP64 transforms (dft.cu): the inputs of the U-matrix product
 bie_status velocity_weights(bie_ctx* c, int nvec, const double* omega, float* xh, float* xl,
                             float2* hw0) {
   const Blocks B = make_blocks(c);
@@ -275,23 +275,15 @@ bie_status velocity_weights(bie_ctx* c, int nvec, const double* omega, float* xh
   double2 *dY, *dX2;
   BIE_GET(c, double2, "mdft_Y", (size_t)nvec * (N + M0), dY);
   BIE_GET(c, double2, "mdft_X2", (size_t)nvec * (N + M0), dX2);
-  bool oom = false;
-  if (oom) return ctx_fail(c, BIE_ERR_OOM, "velocity: twiddles");
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  int s1 = 0, s2 = 0;
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J1.j[J1.n++] = DftJob{M, M1, M / M1, o, o, o, 0, s1};
-    s1 += M;
-    J2.j[J2.n++] = DftJob{M, M1, M / M1, o, o, o, 1, s2};
-    s2 += M;
+    J1.j[J1.n++] = DftJob{M, M1, o, o, o, 0};
+    J2.j[J2.n++] = DftJob{M, M1, o, o, o, 1};
   }
-  J2.j[J2.n++] = DftJob{M0, c->fft_m1[0], M0 / c->fft_m1[0], 0, N, 0, 2, s2};
-  s2 += M0;
-  J1.total = s1;
-  J2.total = s2;
+  J2.j[J2.n++] = DftJob{M0, c->fft_m1[0], 0, N, 0, 2};
   const long long sY = N + M0;
   // every vector's work arrays have stride N + M0; the spectra of the first
   // pair of passes go to X2, which the second pair reads and then overwrites
@@ -360,18 +352,12 @@ bie_status velocity_run(bie_ctx* c, const double* omega, double* U, double* psi,
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  int s1 = 0, s2 = 0;
   for (int k = 0; k < c->nb; ++k) {
     const int M = c->M[k], M1 = c->fft_m1[k], o = c->off[k];
-    J1.j[J1.n++] = DftJob{M, M1, M / M1, o, o, o, 0, s1};
-    s1 += M;
-    J2.j[J2.n++] = DftJob{M, M1, M / M1, o, o, o, 1, s2};
-    s2 += M;
+    J1.j[J1.n++] = DftJob{M, M1, o, o, o, 0};
+    J2.j[J2.n++] = DftJob{M, M1, o, o, o, 1};
   }
-  J2.j[J2.n++] = DftJob{M0, c->fft_m1[0], M0 / c->fft_m1[0], 0, N, 0, 2, s2};
-  s2 += M0;
-  J1.total = s1;
-  J2.total = s2;
+  J2.j[J2.n++] = DftJob{M0, c->fft_m1[0], 0, N, 0, 2};
   if (bie_status sd = dft_run(c, J1, omega, nullptr, dY, dX1)) return sd;
   // inverse of (i k X) per boundary and of (|k| X_0), as conj(DFT(conj(.)))
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
@@ -613,18 +599,12 @@ extern "C" bie_status bie_normal_velocity_static(int nb, const int* M_host, cons
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
-  int s1 = 0, s2 = 0;
   for (int k = 0; k < nb; ++k) {
     const int M = B.M[k], o = B.off[k];
-    J1.j[J1.n++] = DftJob{M, m1[k], M / m1[k], o, o, o, 0, s1};
-    s1 += M;
-    J2.j[J2.n++] = DftJob{M, m1[k], M / m1[k], o, o, o, 1, s2};
-    s2 += M;
+    J1.j[J1.n++] = DftJob{M, m1[k], o, o, o, 0};
+    J2.j[J2.n++] = DftJob{M, m1[k], o, o, o, 1};
   }
-  J2.j[J2.n++] = DftJob{M0, m1[0], M0 / m1[0], 0, (int)N, 0, 2, s2};
-  s2 += M0;
-  J1.total = s1;
-  J2.total = s2;
+  J2.j[J2.n++] = DftJob{M0, m1[0], 0, (int)N, 0, 2};
   if (dft_run_plain(st, J1, omega_dev, nullptr, tw, dY, dX1) != cudaSuccess ||
       dft_run_plain(st, J2, nullptr, dX1, tw, dY, dX2) != cudaSuccess)
     return BIE_ERR_CUDA;
@@ -691,14 +671,13 @@ extern "C" bie_status bie_pressure_rhs(bie_ctx* c, const double* phit, const dou
   const double2* dz64 = (const double2*)ctx_buf(c, "dzeta", sizeof(double2) * N, &oom);
   const double2* d2z64 = (const double2*)ctx_buf(c, "d2zeta", sizeof(double2) * N, &oom);
   if (oom) return ctx_fail(c, BIE_ERR_OOM, "bie_pressure_rhs: buffers");
-  // phi~_alpha by the four-step DFT of the surface block (modes 0 then 1)
+  // phi~_alpha by transforms of the surface block (modes 0 then 1)
   DftJobs J1, J2;
   memset(&J1, 0, sizeof(J1));
   memset(&J2, 0, sizeof(J2));
   const int M1 = c->fft_m1[0];
-  J1.j[J1.n++] = DftJob{M0, M1, M0 / M1, 0, 0, 0, 0, 0};
-  J2.j[J2.n++] = DftJob{M0, M1, M0 / M1, 0, 0, 0, 1, 0};
-  J1.total = J2.total = M0;
+  J1.j[J1.n++] = DftJob{M0, M1, 0, 0, 0, 0};
+  J2.j[J2.n++] = DftJob{M0, M1, 0, 0, 0, 1};
   if (bie_status sd = dft_run(c, J1, phit, nullptr, dY, dX1)) return sd;
   if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   k_pressure_rhs<<<obs_grid(N), NODE_THREADS, 0, c->stream>>>(N, M0, make_flow(c), dX2, z64, dz64, d2z64,

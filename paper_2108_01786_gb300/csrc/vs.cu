@@ -266,9 +266,8 @@ extern "C" bie_status bie_vs_normal_velocity(bie_ctx* c, const double* gamma0, d
     memset(&J1, 0, sizeof(J1));
     memset(&J2, 0, sizeof(J2));
     const int m1 = c->fft_m1[0];
-    J1.j[J1.n++] = DftJob{M0, m1, M0 / m1, 0, 0, 0, 0, 0};
-    J2.j[J2.n++] = DftJob{M0, m1, M0 / m1, 0, 0, 0, 4, 0};
-    J1.total = J2.total = M0;
+    J1.j[J1.n++] = DftJob{M0, m1, 0, 0, 0, 0};
+    J2.j[J2.n++] = DftJob{M0, m1, 0, 0, 0, 4};
     if (bie_status sd = dft_run(c, J1, gamma0, nullptr, dY, dX1)) return sd;
     if (bie_status sd = dft_run(c, J2, nullptr, dX1, dY, dX2)) return sd;
   }
