@@ -50,7 +50,8 @@ def _peaks():
 
 # the source files that define each profiled kernel
 KERNEL_SOURCES = {
-    "k_gemv_lowp": ("gemv.cu", "gemv_dot.cuh", "common.cuh"),
+    "k_resident": ("resident.cu", "gemv_dot.cuh", "tfl.h", "krylov.cuh", "common.cuh"),
+    "k_gemv_lowp": ("gemv.cu", "gemv_dot.cuh", "tfl.h", "common.cuh"),
     "k_targets_far": ("targets.cu", "pair_kernel.cuh", "df2.cuh", "common.cuh"),
     "k_targets_helsing": ("targets.cu", "pair_kernel.cuh", "df2.cuh", "common.cuh"),
     "k_assemble_pairs": ("assemble.cu", "pair_kernel.cuh", "df2.cuh", "common.cuh"),
@@ -571,7 +572,8 @@ def run_ours(args):
     roofline = {"bound": "hbm",
                 "kernel": f"k_resident<{tname}>" if one_kernel else STEPWISE,
                 "achieved": achieved_solve, "peak": hb_peak, "peak_kind": peak_kind, "unit": "GB/s",
-                "frac": achieved_solve / hb_peak, "traffic": None,
+                "frac": achieved_solve / hb_peak,
+                "traffic": _traffic(f"k_resident<{tname}>") if one_kernel else None,
                 "avg_launch_ms": solve_ms, "launches": args.steps if one_kernel else None,
                 "algorithmic_bytes_per_launch": solve_bytes,
                 "iters": solve_info.iters, "same_steps_as_counted": solve_info.iters == infos_prof[-1].iters,
