@@ -58,7 +58,7 @@ KERNEL_SOURCES = {
 }
 # FP32 issue peak: 152 SMs x 4 schedulers x 1 warp instruction per cycle
 ISSUE_SLOTS_PER_CYCLE = 152 * 4
-# FP64 FMA throughput measured on this machine's GB300: eight independent DFMA
+# FP64 FMA throughput measured on the GB300: eight independent DFMA
 # chains per thread, 4 x 152 CTAs of 512 threads, CUDA events (1.181-1.196
 # TFLOP/s over three runs; nominal 1.25; the FP32 FMA rate measured the same way
 # is 74.6 TFLOP/s, 62x)
