@@ -64,15 +64,21 @@ __global__ void __launch_bounds__(1024, 1)
       xs4[c] = o;
     }
   }
-  if (mwarp) {
-    double t = 0.0;
+  if (mwarp) {   // obstacles past the CTA's warps (20 to 32) in further rounds
+    for (int o = warp;;) {
+      double t = 0.0;
 #pragma unroll
-    for (int q = 0; q < BIE_NPART / 32; ++q) t += pv[q];
-    t = warp_sum(t);
-    const double mu = t * (double)df.invM[warp];
-    if (lane == 0) {
-      s_xc[warp] = (float)((double)df.coef * mu);
-      if (blockIdx.x == 0 && df.mean_out) df.mean_out[warp] = mu;
+      for (int q = 0; q < BIE_NPART / 32; ++q) t += pv[q];
+      t = warp_sum(t);
+      const double mu = t * (double)df.invM[o];
+      if (lane == 0) {
+        s_xc[o] = (float)((double)df.coef * mu);
+        if (blockIdx.x == 0 && df.mean_out) df.mean_out[o] = mu;
+      }
+      o += (int)(blockDim.x >> 5);
+      if (o >= df.nobs) break;
+#pragma unroll
+      for (int q = 0; q < BIE_NPART / 32; ++q) pv[q] = df.part[(size_t)o * BIE_PSTRIDE + lane + 32 * q];
     }
   }
   __syncthreads();

@@ -264,3 +264,33 @@ def test_option_sets_that_must_converge_and_that_must_not(P, M0, M1, Mo, prec):
             assert 1e-13 < max(res) < 1.0 and max(res) <= 2.0 * min(res), (kw, res)
     finally:
         prob.close()
+
+
+def _many(nobs, M0, M1, Mo):
+    surf = W.fourier_graph(M0, 0.0, np.array([0.08, 0.02]), np.array([0.03, 0.0]))
+    bot = W.graph_curve(M1, lambda a: -1.0 + 0 * a, lambda a: 0 * a, lambda a: 0 * a)
+    r = 1.2 / nobs
+    ells = [(6.28 * (j + 0.5) / nobs, -0.5, r, 0.8 * r, 0.4 * j) for j in range(nobs)]
+    g = W.assemble_geometry([surf, bot] + [W.ellipse(m, *e) for m, e in zip(Mo, ells)], ells)
+    return g, W.Flow(V1=0.7, a=np.linspace(-0.4, 0.5, nobs)), W.filtered_noise(np.random.default_rng(M0), M0, 0.05, 8)
+
+
+@pytest.mark.parametrize("nobs", [19, 20, 25, 30])
+@pytest.mark.parametrize("prec", ["fp32_ir", "bf16_ir"])
+def test_many_obstacles_in_the_kernel_by_kernel_solver(P, nobs, prec):
+    """As many obstacles as boundaries are allowed: the product has 20 to 32 warps, fewer
+    than the obstacles where its chunk of rows needs no more."""
+    import torch
+    g, f, ph = _many(nobs, 100, 60, [16 + j % 5 for j in range(nobs)])
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        b = torch.empty(g.N, dtype=torch.float64, device="cuda")
+        P.bie_rhs(prob.ctx, prob.phit, b)
+        for kw in ({}, {"row_flip": 0}):
+            (s0, x0, i0), (s1, x1, i1) = _both_solvers(P, prob, b, g.N, **kw)
+            assert (s0, s1) == (0, 0) and i0.converged and i1.converged, kw
+            assert abs(i0.iters - i1.iters) <= 3
+            assert float((x0 - x1).norm() / x1.norm()) <= 1e-12
+    finally:
+        prob.close()
