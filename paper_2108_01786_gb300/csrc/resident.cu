@@ -1016,9 +1016,11 @@ __global__ void __launch_bounds__(1024, 1) k_resident(const __grid_constant__ Rs
           constexpr int LN = RC ? 16 : 32;
           const int nd = all ? n3 : nb + 1;
           typename A3::X ld3[A3::LD];
-          // an obstacle's sum (three words) goes to a warp that has none of the first rows
+          // an obstacle's sum (three words) goes to a warp that has none of the first rows; with
+          // more obstacles than warps they are all taken in rounds below
           const int ob = nrw - 1 - warp;
-          const bool mine = !all && ob < nobs && 2 * warp >= nd && nd <= nrt / LN && G <= 32 * A3::LD / 2;
+          const bool mine = !all && ob < nobs && nobs <= nrw && 2 * warp >= nd && nd <= nrt / LN &&
+                            G <= 32 * A3::LD / 2;
           if constexpr (!all) {
             if (mine) {
 #pragma unroll

@@ -294,3 +294,23 @@ def test_many_obstacles_in_the_kernel_by_kernel_solver(P, nobs, prec):
             assert float((x0 - x1).norm() / x1.norm()) <= 1e-12
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("nobs,M0,M1,Mo", [(25, 2400, 1200, 48), (30, 2500, 1300, 46), (30, 60, 40, 20), (21, 2400, 1200, 57)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32_ir", "fp16_ir"])
+def test_more_obstacles_than_row_warps(P, nobs, M0, M1, Mo, prec):
+    """4700 to 5200 unknowns: 32 to 35 rows on 20 to 31 row warps per CTA, fewer than the
+    obstacles whose sums they reduce (21, 25, 30); a small case with more warps than those."""
+    import torch
+    g, f, ph = _many(nobs, M0, M1, [Mo + j % 3 for j in range(nobs)])
+    prob = P.Problem(g, f, ph)
+    try:
+        prob.assemble(prec)
+        b = torch.empty(g.N, dtype=torch.float64, device="cuda")
+        P.bie_rhs(prob.ctx, prob.phit, b)
+        for kw in ({}, {"row_flip": 0}):
+            (s0, x0, i0), (s1, x1, i1) = _both_solvers(P, prob, b, g.N, **kw)
+            assert (s0, s1) == (0, 0) and i0.converged and i1.converged, kw
+            assert float((x0 - x1).norm() / x1.norm()) <= 1e-12
+    finally:
+        prob.close()
