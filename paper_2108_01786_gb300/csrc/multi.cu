@@ -660,15 +660,15 @@ __global__ void k_m_finish_dots(MArgs a, int j, const float* __restrict__ Yp, in
   slice_of(a.N, r0, r1);
   {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < a.nobs) {   // means of v_j over the obstacles, in a fixed order
-      const double* prow = a.part3 + ((size_t)rr * BIE_MAXB + warp) * BIE_PSTRIDE;
+    for (int o = warp; o < a.nobs; o += (int)(blockDim.x >> 5)) {   // means of v_j over the obstacles, in a fixed order
+      const double* prow = a.part3 + ((size_t)rr * BIE_MAXB + o) * BIE_PSTRIDE;
       double t = 0.0;
       for (int q = lane; q < (int)gridDim.x; q += 32) t += prow[q];
       t = warp_sum(t);
-      const double mu = t * a.obs_invM[warp];
+      const double mu = t * a.obs_invM[o];
       if (lane == 0) {
-        s_xc[warp] = (float)(1.5 * mu);
-        if (blockIdx.x == 0) a.mu[((size_t)rr * (a.m + 1) + j) * BIE_MAXB + warp] = mu;
+        s_xc[o] = (float)(1.5 * mu);
+        if (blockIdx.x == 0) a.mu[((size_t)rr * (a.m + 1) + j) * BIE_MAXB + o] = mu;
       }
     }
     __syncthreads();

@@ -338,3 +338,31 @@ def test_repeated_solves_give_the_same_bits(P, n, nrhs):
             assert steps == first[2] and torch.equal(om, first[0]) and torch.equal(U, first[1])
     finally:
         prob.close()
+
+
+@pytest.mark.parametrize("nobs", [7, 8, 9, 17, 30])
+def test_solve_multi_with_many_obstacles(P, nobs):
+    """More obstacles than a Gram-Schmidt CTA has warps (8): every column converges in as many
+    steps as a single solve and to the same solution."""
+    import torch
+    surf = W.fourier_graph(300, 0.0, np.array([0.08, 0.02]), np.array([0.03, 0.0]))
+    bot = W.graph_curve(180, lambda a: -1.0 + 0 * a, lambda a: 0 * a, lambda a: 0 * a)
+    r = min(0.12, 1.2 / nobs)
+    ells = [(6.28 * (j + 0.5) / nobs, -0.5, r, 0.8 * r, 0.4 * j) for j in range(nobs)]
+    g = W.assemble_geometry([surf, bot] + [W.ellipse(24 + j % 5, *e) for j, e in enumerate(ells)], ells)
+    f = W.Flow(V1=0.7, a=np.linspace(-0.4, 0.5, nobs))
+    PH = np.stack([W.filtered_noise(np.random.default_rng(k), g.M[0], 0.05, 6 + k) for k in range(3)])
+    prob = P.Problem(g, f, PH[0])
+    try:
+        prob.assemble("fp16_ir")
+        om = torch.empty((3, g.N), dtype=torch.float64, device="cuda")
+        U = torch.empty((3, g.M[0]), dtype=torch.float64, device="cuda")
+        infos = P.bie_solve_multi(prob.ctx, torch.as_tensor(PH, device="cuda").contiguous(), om, U)
+        x, u = torch.empty_like(om[0]), torch.empty_like(U[0])
+        for k in range(3):
+            one = P.bie_solve(prob.ctx, torch.as_tensor(PH[k], device="cuda"), x, u)
+            assert infos[k].converged and abs(infos[k].iters - one.iters) <= 4, (infos[k].iters, one.iters)
+            assert float((om[k] - x).norm() / x.norm()) <= 1e-12
+            assert float((U[k] - u).norm() / u.norm()) <= 1e-10
+    finally:
+        prob.close()
